@@ -23,6 +23,15 @@ constexpr unsigned kPollSuspendNs = 1000;
 // Device status codes written to the plan's error word.
 constexpr int kDevErrTmaTimeout = 1;
 
+// Wait until every kernel this one was launched behind (launch_chained) has
+// finished and its writes are visible.  A kernel calls it before its first
+// access to global memory, with all its threads; launched any other way it
+// returns at once.
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ uint32_t smem_addr(const void *p)
 {
     return (uint32_t)__cvta_generic_to_shared(p);

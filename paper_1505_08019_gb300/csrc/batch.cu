@@ -81,8 +81,7 @@ cudaError_t batch_launch_h16(BatchTableH16 &t, cudaStream_t s)
         if (e != cudaSuccess)
             return e;
     }
-    k<<<ctas, C::T, SMEM, s>>>(t);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)ctas, C::T, SMEM, s, 1, t);
 }
 
 // The single-image half2 passes' CTA shapes (kernels_h16.cu): rows as for
@@ -116,8 +115,7 @@ cudaError_t batch_launch(BatchTable &t, cudaStream_t s)
         if (e != cudaSuccess)
             return e;
     }
-    k<<<ctas, C::T, C::SMEM_BYTES, s>>>(t);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)ctas, C::T, C::SMEM_BYTES, s, 1, t);
 }
 
 // Grouped persistent TMA column pass: a load and a store tensor map per
@@ -175,9 +173,8 @@ cudaError_t batch_launch_tma(const BatchTable &t, int *err, cudaStream_t s, bool
     int grid = device_sm_count() * occ.get(d);
     if (grid > tiles)
         grid = tiles;
-    k<<<grid, C::T, SMEM, s>>>(tt, t.job[0].tw, err);
     *used = true;
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, tt, t.job[0].tw, err);
 }
 
 template <int L>

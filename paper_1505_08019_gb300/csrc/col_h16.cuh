@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(C::T, 1) col_h16_tma_kernel(const __grid_const
     const int ntiles = cols / C::W;
     const int tid = threadIdx.x;
     int tile = blockIdx.x;
+    pdl_wait();
     if (tid == 0) {
         mbar_init(&bar_early, 1);
         mbar_init(&bar_late, 1);

@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(C::T, C::MINB) line_dct_kernel(const DctIO d,
     extern __shared__ float2 sm[];
     using G0 = Grp<C, 0>;
     const int tid = threadIdx.x;
+    pdl_wait();
     const long long line0 = (long long)blockIdx.x * (ROW ? C::LB : C::W);
     const long long nvalid = nlines - line0;
     float2 a[C::EPT];
@@ -281,6 +282,7 @@ __global__ void __launch_bounds__(C::T, C::MINB) line_idct_kernel(const DctIO d,
     extern __shared__ float2 sm[];
     constexpr int HALF = C::N / 2;
     const int tid = threadIdx.x;
+    pdl_wait();
     const long long line0 = (long long)blockIdx.x * (ROW ? C::LB : C::W);
     const long long nvalid = nlines - line0;
     for (int e = tid; e < C::E; e += C::T) {
@@ -412,8 +414,7 @@ cudaError_t idct_launch(const DctIO &d, const float2 *tw, const float2 *post, lo
     }
     const long long per = ROW ? C::LB : C::W;
     const unsigned grid = (unsigned)((nlines + per - 1) / per);
-    k<<<grid, C::T, bytes, s>>>(d, tw, post, nlines, scale);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, bytes, s, 1, d, tw, post, nlines, scale);
 }
 
 // The last stage group of a line: unit lo (0 <= lo < M = 2^S0) holds rows
@@ -604,6 +605,7 @@ __global__ void __launch_bounds__(C::T, C::MINB) row_dct_kernel(const DctIO d,
     static_assert(HH * C::LB == C::T && P * C::LB == C::T, "threads cover the line blocks");
     extern __shared__ float2 sm[];
     const int tid = threadIdx.x;
+    pdl_wait();
     const long long line0 = (long long)blockIdx.x * C::LB;
     const long long nvalid = nlines - line0;
     float2 a[C::EPT];
@@ -691,8 +693,7 @@ cudaError_t row_dct_launch(const DctIO &d, const float2 *tw, const float2 *post,
             return e;
     }
     const unsigned grid = (unsigned)((nlines + C::LB - 1) / C::LB);
-    k<<<grid, C::T, bytes, s>>>(d, tw, post, dct_rot_table(), nlines, scale);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, bytes, s, 1, d, tw, post, dct_rot_table(), nlines, scale);
 }
 
 // ---------------------------------------------------------------------------
@@ -750,6 +751,7 @@ __global__ void __launch_bounds__(C::T, 1) col_dct_tma_kernel(
     extern __shared__ __align__(1024) float2 sm[];
     __shared__ __align__(8) uint64_t bar_even, bar_odd;
     const int tid = threadIdx.x;
+    pdl_wait();
     int tile = blockIdx.x;
     float2 *pref = sm + C::E;          // even region
     float2 *stw = sm + D::TW_OFF;      // rotation factors, loaded once
@@ -916,9 +918,7 @@ cudaError_t dct_col_tma_launch(const DctIO &d, const float2 *tw, const float2 *p
     int grid = device_sm_count();
     if (grid > ntiles)
         grid = ntiles;
-    k<<<grid, C::T, SMEM, s>>>(me, mo, omap, out, cc, ntiles, tw, post, dct_rot_table(), scale,
-                               err, withhold);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, me, mo, omap, out, cc, ntiles, tw, post, dct_rot_table(), scale, err, withhold);
 }
 
 // ---------------------------------------------------------------------------
@@ -951,6 +951,7 @@ __global__ void __launch_bounds__(C::T, 1) col_dct_tma64_kernel(
     __shared__ __align__(8) uint64_t bar_early, bar_late;
     __shared__ float2 rot_base[R / 2];   // (cos, sin)(pi 2^S0 r / (2N)), r < R/2
     const int tid = threadIdx.x;
+    pdl_wait();
     float2 *stw = sm + S::TW_OFF;
     float2 *stage = sm + C::E / 2;
     const int w = tid & (C::W - 1);
@@ -1145,8 +1146,7 @@ cudaError_t dct_col_tma64_launch(const DctIO &d, const float2 *tw, const float2 
     int grid = device_sm_count();
     if (grid > ntiles)
         grid = ntiles;
-    k<<<grid, C::T, SMEM, s>>>(me, mo, omap, ntiles, tw, post, scale, err, withhold);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, me, mo, omap, ntiles, tw, post, scale, err, withhold);
 }
 
 // ---------------------------------------------------------------------------
@@ -1176,6 +1176,7 @@ __global__ void __launch_bounds__(C::T, 1) col_idct_tma64_kernel(
     __shared__ __align__(8) uint64_t bar_early, bar_late;
     __shared__ float2 rot_top[G0::R];   // (cos, sin)(pi top(r) / (2N)), top(r) = rev(r) 2^HB
     const int tid = threadIdx.x;
+    pdl_wait();
     float2 *stw = sm + S::TW_OFF;
     float2 *stage = sm + C::E / 2;
     const float2 *pref = sm + C::E;
@@ -1331,8 +1332,7 @@ cudaError_t idct_col_tma64_launch(const DctIO &d, const float2 *tw, const float2
     int grid = device_sm_count();
     if (grid > ntiles)
         grid = ntiles;
-    k<<<grid, C::T, SMEM, s>>>(map, oe, oo, ntiles, tw, post, scale, err, withhold);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, oe, oo, ntiles, tw, post, scale, err, withhold);
 }
 
 // ---------------------------------------------------------------------------
@@ -1589,8 +1589,7 @@ cudaError_t dct_launch(const DctIO &d, const float2 *tw, const float2 *post, lon
     }
     const long long per = ROW ? C::LB : C::W;
     const unsigned grid = (unsigned)((nlines + per - 1) / per);
-    k<<<grid, C::T, bytes, s>>>(d, tw, post, nlines, scale);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, bytes, s, 1, d, tw, post, nlines, scale);
 }
 
 // ---------------------------------------------------------------------------
@@ -1669,6 +1668,7 @@ __global__ void __launch_bounds__(C::T, C::MINB) row_idct_kernel(const DctIO d,
     static_assert(HH * C::LB == C::T && P * C::LB == C::T, "threads cover the line blocks");
     extern __shared__ float2 sm[];
     const int tid = threadIdx.x;
+    pdl_wait();
     const long long line0 = (long long)blockIdx.x * C::LB;
     const long long nvalid = nlines - line0;
     float2 a[C::EPT];
@@ -1752,8 +1752,7 @@ cudaError_t row_idct_launch(const DctIO &d, const float2 *tw, const float2 *post
             return e;
     }
     const unsigned grid = (unsigned)((nlines + C::LB - 1) / C::LB);
-    k<<<grid, C::T, bytes, s>>>(d, tw, post, dct_rot_table(), nlines, scale);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, bytes, s, 1, d, tw, post, dct_rot_table(), nlines, scale);
 }
 
 // Inverse column pass, persistent and TMA-fed like the complex column pass
@@ -1782,6 +1781,7 @@ __global__ void __launch_bounds__(C::T, 1) col_idct_tma_kernel(
     extern __shared__ __align__(1024) float2 sm[];
     __shared__ __align__(8) uint64_t bar_early, bar_late;
     const int tid = threadIdx.x;
+    pdl_wait();
     int tile = blockIdx.x;
     const float2 *pref = sm + C::E;
     float2 *stw = sm + S::TW_OFF;
@@ -1935,6 +1935,7 @@ __global__ void __launch_bounds__(C::T, 1) col_idct_pair_kernel(
     cg::cluster_group cluster = cg::this_cluster();
     const int b = (int)cluster.block_rank();
     const int tid = threadIdx.x;
+    pdl_wait();
     const int nclusters = (int)gridDim.x / 2;
     const CUtensorMap *lmap = b == 0 ? &m0 : &m1;
     float2 *stw = sm + S::TW_OFF;
@@ -2228,9 +2229,7 @@ cudaError_t idct_col_tma_launch(const DctIO &d, const float2 *tw, const float2 *
     int grid = device_sm_count();
     if (grid > ntiles)
         grid = ntiles;
-    k<<<grid, C::T, SMEM, s>>>(map, oe, out, cc, ntiles, tw, post, dct_rot_table(), scale, err,
-                               withhold);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, oe, out, cc, ntiles, tw, post, dct_rot_table(), scale, err, withhold);
 }
 
 template <int L>

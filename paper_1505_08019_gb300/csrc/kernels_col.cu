@@ -130,8 +130,8 @@ cudaError_t col_launch(const PassArgs &a, cudaStream_t s)
             return e;
     }
     const unsigned grid = (unsigned)((a.cols + C::W - 1) / C::W);
-    k<<<grid, C::T, dev_bytes, s>>>(StoreC64{a.in, a.out}, a.tw, a.cols, a.ld, a.scale, a.nst);
-    return cudaGetLastError();
+    return launch_chained(k, grid, C::T, dev_bytes, s, 1, StoreC64{a.in, a.out}, a.tw, a.cols, a.ld,
+                          a.scale, a.nst);
 }
 
 template <class C>
@@ -183,9 +183,8 @@ cudaError_t col_launch_tma(const PassArgs &a, cudaStream_t s)
     int grid = sm_count() * occ.get(d);
     if (grid > ntiles)
         grid = ntiles;
-    k<<<grid, C::T, SMEM, s>>>(map, omap, a.out, a.tw, a.cols, a.ld, a.scale, a.err,
-                               a.withhold);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, omap, a.out, a.tw, a.cols, a.ld,
+                          a.scale, a.err, a.withhold);
 }
 
 // Persistent column pass with the next tile parked in TMEM (col_tmem_kernel):

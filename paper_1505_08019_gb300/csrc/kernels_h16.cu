@@ -31,8 +31,7 @@ cudaError_t h16_launch_axis(const H16PassArgs &a, cudaStream_t s)
     const int per = ROW ? C::LB : C::W;
     const unsigned grid = (unsigned)((lines + per - 1) / per);
     IO io{a.in, a.out, a.in_exp, a.in_axis, a.out_exp};
-    k<<<grid, C::T, bytes, s>>>(io, a.tw, lines, a.ld, a.scale, a.nst);
-    return cudaGetLastError();
+    return launch_chained(k, grid, C::T, bytes, s, 1, io, a.tw, lines, a.ld, a.scale, a.nst);
 }
 
 // The input's exponent axis becomes a compile-time choice, so a line's
@@ -100,9 +99,8 @@ cudaError_t h16_launch_col_tma(const H16PassArgs &a, cudaStream_t s)
     int grid = device_sm_count();
     if (grid > ntiles)
         grid = ntiles;
-    k<<<grid, C::T, H::SMEM_BYTES, s>>>(map, omap, a.tw, a.in_exp, a.out_exp, a.cols, a.scale,
-                                        a.err);
-    return cudaGetLastError();
+    return launch_chained(k, (unsigned)grid, C::T, H::SMEM_BYTES, s, 1, map, omap, a.tw, a.in_exp,
+                          a.out_exp, a.cols, a.scale, a.err);
 }
 
 // Columns of 2^(12+CL) rows on a cluster of 2^CL CTAs (col_group_l2_kernel,
@@ -221,6 +219,7 @@ __global__ void h16_pack_kernel(const float2 *in, __half2 *out, int *exp_rows, i
     if (threadIdx.x == 0)
         smax = 0;
     __syncthreads();
+    pdl_wait();
     float m = 0.f;
     for (int i = threadIdx.x; i < cols; i += blockDim.x) {
         const float2 v = src[i];
@@ -242,6 +241,7 @@ __global__ void h16_unpack_kernel(const __half2 *in, const int *exps, int axis, 
                                   int rows, int cols)
 {
     const long long n = (long long)rows * cols;
+    pdl_wait();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
         const long long r = k / cols, c = k - r * cols;
@@ -277,8 +277,7 @@ cudaError_t launch_pass_h16(bool row, int L, const H16PassArgs &a, cudaStream_t 
 cudaError_t launch_h16_pack(const float2 *in, __half2 *out, int *exp_rows, int rows, int cols,
                             cudaStream_t s)
 {
-    h16_pack_kernel<<<rows, 256, 0, s>>>(in, out, exp_rows, cols);
-    return cudaGetLastError();
+    return launch_chained(h16_pack_kernel, (unsigned)rows, 256, 0, s, 1, in, out, exp_rows, cols);
 }
 
 cudaError_t launch_h16_unpack(const __half2 *in, const int *exps, int axis, float2 *out,
@@ -288,8 +287,8 @@ cudaError_t launch_h16_unpack(const __half2 *in, const int *exps, int axis, floa
     long long blocks = (n + 255) / 256;
     if (blocks > 4096)
         blocks = 4096;
-    h16_unpack_kernel<<<(unsigned)blocks, 256, 0, s>>>(in, exps, axis, out, rows, cols);
-    return cudaGetLastError();
+    return launch_chained(h16_unpack_kernel, (unsigned)blocks, 256, 0, s, 1, in, exps, axis, out, rows,
+                          cols);
 }
 
 }  // namespace fft2d

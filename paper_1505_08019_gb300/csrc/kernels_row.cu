@@ -33,8 +33,8 @@ cudaError_t row_launch(const PassArgs &a, cudaStream_t s)
             return e;
     }
     const unsigned grid = (unsigned)((a.rows + C::LB - 1) / C::LB);
-    k<<<grid, C::T, dev_bytes, s>>>(StoreC64{a.in, a.out}, a.tw, a.rows, a.ld, a.scale, a.nst);
-    return cudaGetLastError();
+    return launch_chained(k, grid, C::T, dev_bytes, s, 1, StoreC64{a.in, a.out}, a.tw, a.rows, a.ld,
+                          a.scale, a.nst);
 }
 
 template <class C>

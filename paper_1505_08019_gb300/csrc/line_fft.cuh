@@ -556,6 +556,7 @@ __device__ __forceinline__ void line_fft(const IO &io, const Geo &g,
         if constexpr (C::NG == 1)
             __syncthreads();
     }
+    pdl_wait();
     float2 a[C::EPT];
     group_first<C, ROW, GENERIC, IO>(a, sm, io, g, tw, scale, nst, nvalid, sred);
     if constexpr (C::NG >= 2) {
@@ -1092,6 +1093,7 @@ __device__ __forceinline__ void col_tma2_body(const Src &src, int ntiles,
         fence_mbar_init();
     }
     __syncthreads();
+    pdl_wait();
     // the rotation factors (N entries, the last one padding) stay in shared
     // memory for the CTA's whole life; they arrive with the first tile
     float2 *stw = sm + TmaSplit<C>::TW_OFF;

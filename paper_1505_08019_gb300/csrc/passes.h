@@ -20,6 +20,38 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// Launch of a kernel that begins with pdl_wait() (async_copy.cuh), allowed to
+// start while the previous kernel of the stream is still draining
+// (programmatic stream serialisation): its launch and set-up overlap that
+// kernel's tail and write-back, and pdl_wait() orders everything after them.
+// Back to back on a GB300, empty kernels follow one another every 0.5 us
+// (CUDA graph) to 1.4 us (stream, host bound) this way, against 2.1 us; a
+// 1024^2 inverse transform takes 10.2 instead of 14.3 us, a 4096^2 forward
+// one 98.8 instead of 103.5, a 4096^2 DCT 65.6 instead of 70.0.  The
+// successor is let in only when this kernel's CTAs have left (no early
+// trigger), so its waiting CTAs never hold room another stream could use.
+// cluster > 1: clusters of that many CTAs.
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*k)(P...), dim3 grid, unsigned block, size_t smem,
+                                  cudaStream_t s, unsigned cluster, A &&...args)
+{
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<A &&>(args)...);
+}
+
 // One int per device (index from device_current(), below 64), computed on
 // first use by the launching thread; threads that race on the first use
 // compute and store the same value.
