@@ -73,7 +73,7 @@ template <class C>
 __global__ void __launch_bounds__(C::T, 1) col_h16_tma_kernel(const __grid_constant__ CUtensorMap map,
                                                               const __grid_constant__ CUtensorMap omap,
                                                               const float2 *__restrict__ tw,
-                                                              const int *__restrict__ row_exp,
+                                                              const int *row_exp,
                                                               int *out_exp, int cols, float scale,
                                                               int *err)
 {

@@ -68,10 +68,10 @@ __device__ __forceinline__ float2 dct_load(const DctIO &d, long long line0, int 
     const int s = dct_src(i, C::N);
     if constexpr (ROW) {
         const long long ra = 2 * (line0 + lb);
-        return make_float2(__ldg(d.in + ra * d.cols + s), __ldg(d.in + (ra + 1) * d.cols + s));
+        return make_float2(ld_img(d.in + ra * d.cols + s), ld_img(d.in + (ra + 1) * d.cols + s));
     } else {
         const float2 *p = reinterpret_cast<const float2 *>(d.in);
-        return __ldg(p + (long long)s * (d.cols / 2) + line0 + w);
+        return ld_img(p + (long long)s * (d.cols / 2) + line0 + w);
     }
 }
 
@@ -293,9 +293,9 @@ __global__ void __launch_bounds__(C::T, C::MINB) line_idct_kernel(const DctIO d,
         if (ROW ? lb < nvalid : w < nvalid) {
             if constexpr (ROW) {
                 const long long ra = 2 * (line0 + lb);
-                z = make_float2(__ldg(d.in + ra * d.cols + k), __ldg(d.in + (ra + 1) * d.cols + k));
+                z = make_float2(ld_img(d.in + ra * d.cols + k), ld_img(d.in + (ra + 1) * d.cols + k));
             } else {
-                z = __ldg(reinterpret_cast<const float2 *>(d.in) + (long long)k * (d.cols / 2) +
+                z = ld_img(reinterpret_cast<const float2 *>(d.in) + (long long)k * (d.cols / 2) +
                           line0 + w);
             }
         }
@@ -622,10 +622,10 @@ __global__ void __launch_bounds__(C::T, C::MINB) row_dct_kernel(const DctIO d,
             const int rc = r ^ (G0::R - 1);
             float2 fa = make_float2(0.f, 0.f), fb = fa, ga = fa, gb = fa;
             if (ok) {
-                fa = __ldg(reinterpret_cast<const float2 *>(ra + 2 * (top + h)));
-                fb = __ldg(reinterpret_cast<const float2 *>(rb + 2 * (top + h)));
-                ga = __ldg(reinterpret_cast<const float2 *>(ra + 2 * (top + h1)));
-                gb = __ldg(reinterpret_cast<const float2 *>(rb + 2 * (top + h1)));
+                fa = ld_img(reinterpret_cast<const float2 *>(ra + 2 * (top + h)));
+                fb = ld_img(reinterpret_cast<const float2 *>(rb + 2 * (top + h)));
+                ga = ld_img(reinterpret_cast<const float2 *>(ra + 2 * (top + h1)));
+                gb = ld_img(reinterpret_cast<const float2 *>(rb + 2 * (top + h1)));
             }
             a[r] = make_float2(fa.x, fb.x);                  // unit 0, position top + h
             a[G0::R + rc] = make_float2(fa.y, fb.y);         // unit 1, N-1-(top + h)
@@ -1682,8 +1682,8 @@ __global__ void __launch_bounds__(C::T, C::MINB) row_idct_kernel(const DctIO d,
 #pragma unroll
         for (int r = 0; r < G0::R; r++) {
             const int top = brev_c(r, G0::G) << G0::HB;
-            a[r] = ok ? make_float2(__ldg(ra + top + h), __ldg(rb + top + h)) : make_float2(0.f, 0.f);
-            a[G0::R + r] = ok ? make_float2(__ldg(ra + top + h1), __ldg(rb + top + h1))
+            a[r] = ok ? make_float2(ld_img(ra + top + h), ld_img(rb + top + h)) : make_float2(0.f, 0.f);
+            a[G0::R + r] = ok ? make_float2(ld_img(ra + top + h1), ld_img(rb + top + h1))
                               : make_float2(0.f, 0.f);
         }
         idct_pre_units<C>(a, h, post, rot);

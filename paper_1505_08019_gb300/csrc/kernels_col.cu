@@ -130,7 +130,7 @@ cudaError_t col_launch(const PassArgs &a, cudaStream_t s)
             return e;
     }
     const unsigned grid = (unsigned)((a.cols + C::W - 1) / C::W);
-    return launch_chained(k, grid, C::T, dev_bytes, s, 1, StoreC64{a.in, a.out}, a.tw, a.cols, a.ld,
+    return launch_chained(k, grid, C::T, dev_bytes, s, {1, a.chained}, StoreC64{a.in, a.out}, a.tw, a.cols, a.ld,
                           a.scale, a.nst);
 }
 
@@ -183,7 +183,7 @@ cudaError_t col_launch_tma(const PassArgs &a, cudaStream_t s)
     int grid = sm_count() * occ.get(d);
     if (grid > ntiles)
         grid = ntiles;
-    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, omap, a.out, a.tw, a.cols, a.ld,
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, {1, a.chained}, map, omap, a.out, a.tw, a.cols, a.ld,
                           a.scale, a.err, a.withhold);
 }
 

@@ -33,7 +33,7 @@ cudaError_t row_launch(const PassArgs &a, cudaStream_t s)
             return e;
     }
     const unsigned grid = (unsigned)((a.rows + C::LB - 1) / C::LB);
-    return launch_chained(k, grid, C::T, dev_bytes, s, 1, StoreC64{a.in, a.out}, a.tw, a.rows, a.ld,
+    return launch_chained(k, grid, C::T, dev_bytes, s, {1, a.chained}, StoreC64{a.in, a.out}, a.tw, a.rows, a.ld,
                           a.scale, a.nst);
 }
 

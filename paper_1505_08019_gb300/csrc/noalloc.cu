@@ -117,6 +117,7 @@ fft2d_status fft2d_exec_noalloc(int rows, int cols, int dir, const void *in, voi
     a.ld = cols;
     a.err = &scratch->status;
     a.partial = false;
+    a.chained = false;   // the tables come from the kernel launched just above
     const float inv_scale = (float)(1.0 / ((double)rows * (double)cols));
     // row pass: in -> out (a length-1 row is the identity)
     if (Lc == 0) {

@@ -30,25 +30,39 @@ struct NvtxRange {
 // one 98.8 instead of 103.5, a 4096^2 DCT 65.6 instead of 70.0.  The
 // successor is let in only when this kernel's CTAs have left (no early
 // trigger), so its waiting CTAs never hold room another stream could use.
+// What such a kernel reads through the read-only path, or through a
+// __restrict__ const pointer, may be fetched before the wait: only a plan's
+// tables are read so, never image data, and chained = false is for callers
+// whose tables the previous kernel has just written.
 // cluster > 1: clusters of that many CTAs.
+struct LaunchHow {
+    unsigned cluster;
+    bool chained;
+    LaunchHow(unsigned cluster_ = 1, bool chained_ = true) : cluster(cluster_), chained(chained_) {}
+};
 template <class... P, class... A>
 inline cudaError_t launch_chained(void (*k)(P...), dim3 grid, unsigned block, size_t smem,
-                                  cudaStream_t s, unsigned cluster, A &&...args)
+                                  cudaStream_t s, LaunchHow how, A &&...args)
 {
     cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = cluster;
-    at[1].val.clusterDim.y = 1;
-    at[1].val.clusterDim.z = 1;
+    unsigned n = 0;
+    if (how.chained) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (how.cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = how.cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n++].val.clusterDim.z = 1;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = at;
-    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, k, static_cast<A &&>(args)...);
 }
 
@@ -75,6 +89,7 @@ struct PassArgs {
     int *err;            // device status word (bounded-wait timeouts)
     int variant = -1;    // kernel variant index (-1: the default for this size)
     int withhold = 0;    // self-test: CTA 0 does not issue its first tile's second TMA load
+    bool chained = true; // tw was written before the kernel just ahead on the stream (launch_chained)
 };
 
 // One way to run a pass for one line length (see kernels_row.cu and
