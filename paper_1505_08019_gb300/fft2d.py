@@ -164,6 +164,11 @@ def _hptr(x) -> int:
 def _stream(s) -> int:
     if s is None:
         import torch
+        # the raw handle of torch.cuda.current_stream() without building the
+        # Stream object: 0.4 us instead of 3.0 of a call's host time
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None and torch.cuda.is_initialized():
+            return raw(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(s, int):
         return s
