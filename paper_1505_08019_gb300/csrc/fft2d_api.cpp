@@ -241,6 +241,12 @@ fft2d_status run_dct_pass(const fft2d_plan_s *p, int pass, const void *in, void 
     return FFT2D_OK;
 }
 
+fft2d::SmallArgs small_args(const fft2d_plan_s *p)
+{
+    return {p->tw_rows, p->tw_cols, p->Lr, p->Lc,
+            p->dir == FFT2D_INVERSE ? (float)(1.0 / ((double)p->rows * (double)p->cols)) : 1.0f};
+}
+
 fft2d_status exec_impl(const fft2d_plan_s *p, const void *in, void *out, int rs, int cs,
                        cudaStream_t st)
 {
@@ -251,6 +257,16 @@ fft2d_status exec_impl(const fft2d_plan_s *p, const void *in, void *out, int rs,
         return run_dct_pass(p, FFT2D_PASS_COLS, out, out, st);
     }
     const bool full = (rs < 0 || rs == p->Lc) && (cs < 0 || cs == p->Lr);
+    // default plans of small images: one launch (a forced or tuned pass
+    // variant is a choice of two-launch kernels and is kept)
+    if (full && p->row_variant < 0 && p->col_variant < 0 && fft2d::small_image(p->Lr, p->Lc)) {
+        fft2d::NvtxRange range("fft2d small image");
+        const cudaError_t e =
+            fft2d::launch_small(small_args(p), static_cast<const float2 *>(in),
+                                static_cast<float2 *>(out), st);
+        if (e != cudaErrorNotSupported)
+            return e == cudaSuccess ? FFT2D_OK : cuda_fail(e, "small image launch");
+    }
     fft2d_status s = run_pass(p, FFT2D_PASS_ROWS, in, out, rs, full, st);
     if (s != FFT2D_OK)
         return s;
@@ -868,6 +884,36 @@ fft2d_status fft2d_autotune(fft2d_plan_t p, void *stream)
             save_tune_file_locked();
         }
     }
+    // a small image may be faster in its one launch than with the winners:
+    // then the plan goes back to the defaults, which take it
+    if (e == cudaSuccess && p->dtype == FFT2D_C64 && fft2d::small_image(p->Lr, p->Lc)) {
+        const fft2d_plan_s tuned = *p;
+        fft2d_plan_s plain = *p;
+        plain.row_variant = plain.col_variant = -1;
+        const fft2d_plan_s *side[2] = {&tuned, &plain};
+        float ms[2] = {0.f, 0.f};
+        for (int k = 0; k < 2 && result == FFT2D_OK && e == cudaSuccess; k++) {
+            for (int r = 0; r < 12 && result == FFT2D_OK && e == cudaSuccess; r++) {
+                if (r == 2)
+                    e = cudaEventRecord(e0, st);
+                if (e == cudaSuccess)
+                    result = exec_impl(side[k], a, b, -1, -1, st);
+            }
+            if (result == FFT2D_OK && e == cudaSuccess)
+                e = cudaEventRecord(e1, st);
+            if (result == FFT2D_OK && e == cudaSuccess)
+                e = cudaEventSynchronize(e1);
+            if (result == FFT2D_OK && e == cudaSuccess)
+                e = cudaEventElapsedTime(&ms[k], e0, e1);
+        }
+        if (result == FFT2D_OK && e == cudaSuccess && ms[1] < ms[0]) {
+            p->row_variant = p->col_variant = -1;
+            std::lock_guard<std::mutex> lock(g_tune_mu);
+            g_tuned.erase(std::make_tuple(p->device, (int)FFT2D_PASS_ROWS, p->Lc, p->rows));
+            g_tuned.erase(std::make_tuple(p->device, (int)FFT2D_PASS_COLS, p->Lr, p->cols));
+            save_tune_file_locked();
+        }
+    }
     if (e != cudaSuccess)
         result = cuda_fail(e, "fft2d_autotune");
     if (e0)
@@ -891,6 +937,13 @@ fft2d_status fft2d_exec_h16(fft2d_plan_t p, const void *in, const int *in_exp, i
     if (s != FFT2D_OK)
         return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (fft2d::small_image(p->Lr, p->Lc)) {
+        const cudaError_t e = fft2d::launch_small_h16(
+            small_args(p), static_cast<const __half2 *>(in), in_exp, in_axis,
+            static_cast<__half2 *>(out), p->exp_rows, out_exp, st);
+        if (e != cudaErrorNotSupported)
+            return e == cudaSuccess ? FFT2D_OK : cuda_fail(e, "small half2 image");
+    }
     fft2d::H16PassArgs a;
     a.rows = p->rows;
     a.cols = p->cols;

@@ -224,6 +224,7 @@ __device__ __forceinline__ void run_stages(float2 (&a)[C::EPT], int v, int lo,
 //    every stored |q| < 2^14, well inside half precision's range.
 struct StoreC64 {
     static constexpr bool H16 = false;
+    static constexpr bool CG = false;   // load through L2 only (see small.cu)
     static constexpr int AXIS = -1;
     using T = float2;
     const float2 *in;
@@ -235,6 +236,7 @@ struct StoreC64 {
 template <int IA = -1>
 struct StoreH16T {
     static constexpr bool H16 = true;
+    static constexpr bool CG = false;
     static constexpr int AXIS = IA;
     using T = __half2;
     const __half2 *in;
@@ -290,6 +292,8 @@ __device__ __forceinline__ float in_factor(const IO &io, const Geo &g, int lb, i
 {
     const long long line = io.axis() == 0 ? (ROW ? g.r0 + lb : g.r0 + (long long)i * g.rstep)
                                           : (ROW ? (long long)i : g.c0 + w);
+    if constexpr (IO::CG)
+        return pow2f(__ldcg(io.in_exp + line));
     return pow2f(io.in_exp[line]);
 }
 
@@ -301,10 +305,17 @@ __device__ __forceinline__ float2 load_pix(const IO &io, const Geo &g, int lb, i
 {
     const long long k = pix<ROW>(g, lb, i, w);
     if constexpr (IO::H16) {
-        const float2 q = __half22float2(io.in[k]);
+        __half2 h;
+        if constexpr (IO::CG)
+            h = __ldcg(io.in + k);
+        else
+            h = io.in[k];
+        const float2 q = __half22float2(h);
         if constexpr (!H16PerUnit<IO, ROW>::value)
             f = in_factor<IO, ROW>(io, g, lb, i, w);
         return make_float2(q.x * f, q.y * f);
+    } else if constexpr (IO::CG) {
+        return __ldcg(io.in + k);
     } else {
         return ld_stream(io.in + k);
     }

@@ -151,6 +151,20 @@ cudaError_t launch_h16_pack(const float2 *in, __half2 *out, int *exp_rows, int r
 cudaError_t launch_h16_unpack(const __half2 *in, const int *exps, int axis, float2 *out,
                               int rows, int cols, cudaStream_t s);
 
+// The whole 2D transform of a small image in one launch (small.cu), the same
+// bits as the two passes.  small_image: whether an image of 2^Lr x 2^Lc
+// qualifies.  cudaErrorNotSupported (nothing launched) where the device
+// cannot hold the cluster.  scale: of the column phase's store.
+struct SmallArgs {
+    const float2 *tw_rows, *tw_cols;
+    int Lr, Lc;
+    float scale;
+};
+bool small_image(int Lr, int Lc);
+cudaError_t launch_small(const SmallArgs &a, const float2 *in, float2 *out, cudaStream_t s);
+cudaError_t launch_small_h16(const SmallArgs &a, const __half2 *in, const int *in_exp, int in_axis,
+                             __half2 *out, int *row_exp, int *out_exp, cudaStream_t s);
+
 // Gaussian low-pass multiply of an unshifted spectrum (filter.cu).
 cudaError_t launch_lowpass(bool half2, void *x, int rows, int cols, float sigma_r, float sigma_c,
                            cudaStream_t s);

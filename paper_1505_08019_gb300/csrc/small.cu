@@ -1,0 +1,155 @@
+// small.cu -- the whole 2D transform of a small image in one launch.
+//
+// Up to 2^16 pixels an image is a few microseconds of launch and latency, not
+// of bandwidth: two launches of 8 to 16 CTAs each.  Here one cluster of at
+// most 16 CTAs holds the image, 4096 values (256 threads x 16) per CTA: every
+// CTA transforms its 4096 / cols rows into `out` (which stays in L2), one
+// cluster barrier orders that before the reads of the column phase, and every
+// CTA transforms its 4096 / rows columns in place.  Both phases are the
+// per-CTA line transforms of the two-launch path, so the results are its
+// results bit for bit.  The axis lengths are chosen at run time inside the
+// kernel (both phases have the same CTA shape whatever the length).
+//
+// What bounds it: the latency of two load - exchange - store chains and the
+// barrier between them.  Measured, calls in a row: a 256^2 forward transform
+// takes 5.0 us against 10.1 in two launches.  Why 4096 values per CTA: the same 64-register,
+// 32 KB configuration serves every axis from 2 to 4096 points, and 16 CTAs
+// spread 2^16 pixels over as many SMs as one cluster may span.
+#include "line_fft.cuh"
+#include "passes.h"
+
+namespace fft2d {
+
+namespace {
+
+constexpr int kSmallL = 12;               // log2 of the values per CTA
+constexpr int kSmallMaxCtas = 16;         // largest cluster (non-portable above 8)
+
+// The column phase reads what other CTAs of the cluster have just written.
+struct StoreC64Shared : StoreC64 {
+    static constexpr bool CG = true;
+};
+template <int IA>
+struct StoreH16Shared : StoreH16T<IA> {
+    static constexpr bool CG = true;
+};
+
+template <int L, bool ROW, class IO>
+__device__ __forceinline__ void small_axis(const IO &io, const float2 *__restrict__ tw, float scale,
+                                           int cta, int lines, int ld)
+{
+    using C = LineCfg<L, ROW ? 0 : kSmallL - L, ROW ? kSmallL - L : 0>;
+    constexpr int PER = 1 << (kSmallL - L);   // lines per CTA
+    const long long l0 = (long long)cta * PER;
+    line_fft<C, ROW, true, IO>(io, ROW ? Geo{l0, 1, 0, ld} : Geo{0, 1, l0, ld}, tw, scale, L,
+                               lines - l0);
+}
+
+template <bool ROW, class IO>
+__device__ __forceinline__ void small_phase(int L, const IO &io, const float2 *__restrict__ tw,
+                                            float scale, int cta, int lines, int ld)
+{
+    switch (L) {
+    case 1: return small_axis<1, ROW>(io, tw, scale, cta, lines, ld);
+    case 2: return small_axis<2, ROW>(io, tw, scale, cta, lines, ld);
+    case 3: return small_axis<3, ROW>(io, tw, scale, cta, lines, ld);
+    case 4: return small_axis<4, ROW>(io, tw, scale, cta, lines, ld);
+    case 5: return small_axis<5, ROW>(io, tw, scale, cta, lines, ld);
+    case 6: return small_axis<6, ROW>(io, tw, scale, cta, lines, ld);
+    case 7: return small_axis<7, ROW>(io, tw, scale, cta, lines, ld);
+    case 8: return small_axis<8, ROW>(io, tw, scale, cta, lines, ld);
+    case 9: return small_axis<9, ROW>(io, tw, scale, cta, lines, ld);
+    case 10: return small_axis<10, ROW>(io, tw, scale, cta, lines, ld);
+    case 11: return small_axis<11, ROW>(io, tw, scale, cta, lines, ld);
+    case 12: return small_axis<12, ROW>(io, tw, scale, cta, lines, ld);
+    }
+}
+
+// One cluster = the whole grid.  rio / cio: the storage of the two phases.
+template <class RIO, class CIO>
+__global__ void __launch_bounds__(256, 4) small_kernel(const RIO rio, const CIO cio,
+                                                       const float2 *__restrict__ tw_rows,
+                                                       const float2 *__restrict__ tw_cols, int rows,
+                                                       int cols, int Lr, int Lc, float scale)
+{
+    const int cta = (int)blockIdx.x;
+    small_phase<true>(Lc, rio, tw_rows, 1.0f, cta, rows, cols);
+    // every row is in `out` before any column is read, and the exchange
+    // buffer is free again
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    small_phase<false>(Lr, cio, tw_cols, scale, cta, cols, cols);
+}
+
+// Exchange buffer of 2^12 values, or (axes of up to 16 points: no exchange)
+// the half2 exponent reduction of up to 2^11 lines; with an exchange, at most
+// 2^7 lines reduce behind it.
+constexpr int kSmallSmem = (1 << kSmallL) * 8 + 128 * 4;
+
+template <class RIO, class CIO>
+cudaError_t small_launch(const RIO &rio, const CIO &cio, const SmallArgs &a, cudaStream_t s)
+{
+    auto k = small_kernel<RIO, CIO>;
+    const int ctas = a.Lr + a.Lc > kSmallL ? 1 << (a.Lr + a.Lc - kSmallL) : 1;
+    if (ctas > 8) {
+        // clusters above 8 CTAs are opt-in, and a device may refuse them
+        static DeviceCache ok;   // 1: usable, 2: not
+        const int d = device_current();
+        if (!ok.get(d)) {
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            int n = 0;
+            if (e == cudaSuccess) {
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = kSmallMaxCtas;
+                at[0].val.clusterDim.y = 1;
+                at[0].val.clusterDim.z = 1;
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3(kSmallMaxCtas);
+                cfg.blockDim = dim3(256);
+                cfg.dynamicSmemBytes = kSmallSmem;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
+            }
+            if (e != cudaSuccess)
+                cudaGetLastError();
+            ok.set(d, e == cudaSuccess && n > 0 ? 1 : 2);
+        }
+        if (ok.get(d) != 1)
+            return cudaErrorNotSupported;
+    }
+    return launch_chained(k, dim3(ctas), 256, kSmallSmem, s, LaunchHow((unsigned)ctas), rio, cio,
+                          a.tw_rows, a.tw_cols, 1 << a.Lr, 1 << a.Lc, a.Lr, a.Lc, a.scale);
+}
+
+}  // namespace
+
+// 2^16 pixels is the most that one cluster holds at 4096 values per CTA.
+bool small_image(int Lr, int Lc)
+{
+    return Lr >= 1 && Lc >= 1 && Lr <= kSmallL && Lc <= kSmallL && Lr + Lc <= kSmallL + 4;
+}
+
+cudaError_t launch_small(const SmallArgs &a, const float2 *in, float2 *out, cudaStream_t s)
+{
+    StoreC64Shared c;
+    c.in = out;
+    c.out = out;
+    return small_launch(StoreC64{in, out}, c, a, s);
+}
+
+cudaError_t launch_small_h16(const SmallArgs &a, const __half2 *in, const int *in_exp, int in_axis,
+                             __half2 *out, int *row_exp, int *out_exp, cudaStream_t s)
+{
+    StoreH16Shared<0> c;
+    c.in = out;
+    c.out = out;
+    c.in_exp = row_exp;
+    c.in_axis = 0;
+    c.out_exp = out_exp;
+    return in_axis == 0 ? small_launch(StoreH16T<0>{in, out, in_exp, 0, row_exp}, c, a, s)
+                        : small_launch(StoreH16T<1>{in, out, in_exp, 1, row_exp}, c, a, s);
+}
+
+}  // namespace fft2d
