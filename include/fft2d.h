@@ -106,11 +106,7 @@ FFT2D_API fft2d_status fft2d_plan(int rows, int cols, int dtype, int dir, fft2d_
  * line (even samples ascending, odd samples descending) followed by a
  * rotation by exp(-i pi k / (2N)) (Makhoul, 1980); the inverse rotates
  * first, then runs the inverse DFT and undoes the reordering.  Two real
- * lines share one complex line, except in the inverse column pass of 16384
- * rows, and in the forward one when cols is not a multiple of 8: there each
- * real column is its own complex line and the pass runs in place (called
- * out of place it first copies `in` to `out` on the stream).  The plan also
- * holds the
+ * lines share one complex line.  The plan also holds the
  * (cos, sin)(pi k / (2N)) tables, built in FP64 and rounded to FP32.
  * Errors: FFT2D_ERR_UNSUPPORTED for a side of 1.  The other entry points
  * reject these plans with FFT2D_ERR_ARG, except fft2d_exec_host,
@@ -142,7 +138,10 @@ FFT2D_API fft2d_status fft2d_selftest_timeout(fft2d_plan_t plan, void *stream);
  * transform into shared memory): runs the plan's column pass over `in` into
  * `out` (device images of the plan's shape and dtype, row pitch = cols;
  * for FFT2D_R32_DCT2 plans the DCT column pass of the plan's direction,
- * which is TMA-fed for columns of 2048 to 16384 points), except that CTA 0
+ * which is TMA-fed for columns of 2048 and 4096 points; plans of 8192 and
+ * 16384 rows whose own column pass waits for nothing on the device -- the
+ * strip kernel, both dtypes -- run the TMA-fed complex64 cluster pass of that
+ * column length instead), except that CTA 0
  * never issues the second TMA load of its
  * first tile.  That CTA's bounded wait gives up after about one second, the
  * kernel records the timeout -- for the cluster kernels of 8192- and
@@ -204,13 +203,14 @@ FFT2D_API fft2d_status fft2d_plan_info(fft2d_plan_t plan, int *rows, int *cols, 
  * load, all log2(cols) stages in one launch), then the column pass (scramble
  * fused, all log2(rows) stages, inverse scale fused into the store).
  * in and out are device pointers to rows*cols pixels; in == out is allowed
- * (in place).  Partial overlap of in and out is not allowed.  Two launches.
+ * (in place).  Partial overlap of in and out is not allowed.  Two launches;
+ * one for images of up to 2^16 pixels with sides of 2 to 4096, several for
+ * the column pass of 8192 and 16384 rows.
  * Once the plan has run on its device (the first launch of each kernel sets
  * its shared-memory limit), the call may be captured in a CUDA graph on
  * `stream`.  It makes no allocation then, except that the column pass of
- * 8192 or 16384 rows (and the DCT column passes of 16384 rows and the
- * forward one of 8192 rows) takes a scratch block (about 20 to 50 MB) for the exchange
- * between the CTAs of a cluster stream-ordered from the library's own
+ * 8192 or 16384 rows (of either dtype) takes a scratch block (at most 64 MiB)
+ * for what its CTAs hand one another stream-ordered from the library's own
  * device memory pool and returns it on `stream` after the launch
  * (cudaMallocFromPoolAsync / cudaFreeAsync: no device synchronisation; the
  * pool keeps its memory, so after the first calls no driver allocation
@@ -223,7 +223,7 @@ FFT2D_API fft2d_status fft2d_exec(fft2d_plan_t plan, const void *in, void *out, 
  * One of the two passes of fft2d_exec: FFT2D_PASS_ROWS reads `in` and writes
  * `out`; FFT2D_PASS_COLS reads `in` and writes `out` and applies the inverse
  * scale.  fft2d_exec(p, x, y) == pass(ROWS, x, y) then pass(COLS, y, y).
- * One launch.
+ * One launch (columns of 8192 and 16384 rows: several).
  */
 FFT2D_API fft2d_status fft2d_exec_pass(fft2d_plan_t plan, int pass, const void *in, void *out,
                              void *stream);
@@ -303,7 +303,7 @@ FFT2D_API fft2d_status fft2d_exec_host_many_async(int n, const fft2d_plan_t *pla
  * group runs the row pass of all its images (a job table travels as a kernel
  * parameter), then one launch per group the column pass -- a handful of
  * launches for any number of images.  Lines of 8192 and 16384 points run
- * each image's single-image pass instead (the cluster column kernels), on
+ * each image's single-image pass instead, on
  * the group's internal stream.  Every image's result is bit for bit the one
  * fft2d_exec gives.  complex64 plans only.
  */

@@ -98,10 +98,6 @@ struct GroupCol {
     // tiles' slots, CS XVALS T values (pair) or CS^2 KEEP_V T (four CTAs)
     static constexpr long long L2_SCRATCH_VALS =
         CL == 2 ? 2LL * CS * CS * KEEP_V * C::T : 2LL * CS * XVALS * C::T;
-    // the mirror exchange of the paired forward DCT per cluster, after the
-    // slots above: per CTA a receive region of CS/2 output blocks, KEEP_V
-    // values per thread each
-    static constexpr long long MIRROR_VALS = (long long)CS * (CS / 2) * KEEP_V * C::T;
     static_assert(C::LB == 1 && ((C::EPT == 32 && C::NG == 3) || (C::EPT == 64 && C::NG == 2)),
                   "512 threads x 32 values in 3 groups, or 256 x 64 in 2");
     static_assert(CL >= 1 && CL <= 2, "two or four CTAs");
@@ -320,22 +316,7 @@ struct GroupH16 {
 struct GroupIO {
     const int *row_exp;
     int *out_exp;
-    float2 *mid_row = nullptr;   // paired forward DCT: output row N/2
 };
-
-// The "two for one" split of Z = DFT(v_a + i v_b) into the DCT-II outputs of
-// the real lines a and b (Makhoul's reduction): from Z[k], Z[k'] (k' = N - k)
-// and (c, s) = (cos, sin)(pi k / (2N)),
-//   xk = (X_a[k], X_b[k]),  xp = (X_a[k'], X_b[k']),  both times scale.
-__device__ __forceinline__ void dct_pair(float2 zk, float2 zp, float2 cs, float scale,
-                                         float2 &xk, float2 &xp)
-{
-    const float c = cs.x * 0.5f * scale, s = cs.y * 0.5f * scale;
-    const float sr = zk.x + zp.x, dr = zp.x - zk.x;   // Zr[k] + Zr[k'], Zr[k'] - Zr[k]
-    const float si = zk.y + zp.y, di = zk.y - zp.y;   // Zi[k] + Zi[k'], Zi[k] - Zi[k']
-    xk = make_float2(c * sr + s * di, c * si + s * dr);     // (X_a[k], X_b[k])
-    xp = make_float2(s * sr - c * di, s * si - c * dr);     // (X_a[k'], X_b[k'])
-}
 
 // C: the local engine; cluster of 2^CL CTAs, this CTA's rank q.  lmap: this
 // CTA's load map (rows CS m + rev_CL(q) of the image; box W x 256 x NB);
@@ -612,53 +593,11 @@ __global__ void __launch_bounds__(C::T, 1) col_group_kernel(const __grid_constan
 // The "lost" flags alternate per tile for the same reason.  xbuf: per
 // cluster of the launch, 2 CS XVALS T values (pair) or 2 CS^2 KEEP_V T
 // (four CTAs), cluster-major; it belongs to this launch alone.
-//
-// DCT == 1: the forward DCT-II of real columns (Section 5's similar transforms;
-// the reduction of a length-N DCT-II to a length-N complex DFT of the
-// reordered line v[j] = x[2j], v[N-1-j] = x[2j+1], X[k] = Re(e^{-i pi k /
-// (2N)} V[k]), Makhoul 1980), one complex line per real column, imaginary
-// part zero: no pairing of outputs (k, N-k) is needed.  A tile is W real
-// columns; CTA q's local line u[m] = v[CS m + rev(q)] is, for m < NL/2, the
-// rows 2 CS m + 2 rev(q) (lmap) and for m >= NL/2 the rows
-// 2 CS (NL-1-m) + 2 CS - 1 - 2 rev(q) read backwards (lmap2: ascending rows
-// 2 CS m' + 2 CS - 1 - 2 rev(q)); both maps have 2-float (8-byte) elements,
-// W/2 per box row.  The outputs X[k] (post = (cos, sin)(pi k / (2N)),
-// k <= N/2) leave as floats through the real output map omap.
-//
-// DCT == 2: the inverse, DCT-III, of real columns, one real line per complex
-// line: V[k] = e^{i pi k / (2N)} (X[k] - i X[N-k]) (X[N] = 0), v = IDFT(V)
-// (the plan's conjugate rotation factors), x[2n] = v[n], x[2n+1] =
-// v[N-1-n].  CTA q's local line holds k = CS m + rev(q), the rows of that
-// residue (lmap, ascending); X[N-k] lies in the rows of residue
-// (CS - rev(q)) mod CS read backwards (lmap2): index NL-1-m, or (NL-m) mod
-// NL for residue 0, where m = 0 takes X[N] = 0.  Outputs n < N/2 go to the
-// even rows (omap: rows 2n'), the others in reverse order to the odd rows
-// (omap2: rows 2n'+1).
-//
-// DCT == 3: the forward DCT-II with two real columns per complex line (the
-// "two for one" split, dct_pair): a tile is W complex = 2W real columns
-// (32-byte rows), the local line is gathered as in DCT == 1 from complex
-// maps (lmap ascending, lmap2 backwards), so half the butterflies of DCT ==
-// 1 per real column.  Output K needs Z[K] and Z[N-K].  CTA q holds K = NL t
-// + k_base + row (row < OUT_ROWS); N - K is row OUT_ROWS - row of block
-// CS-1-t in CTA CS-1-q (k_base(q) + k_base(CS-1-q) = NL - OUT_ROWS), except
-// for row 0, whose mirror is row 0 of the CTA with k_base = NL - k_base(q)
-// (CTA 0 and the CTA at NL/2: itself; CTAs 2 and 3 of four: each other).  So
-// every CTA forms the pairs of its blocks t < CS/2 and sends its blocks t >=
-// CS/2 through a second exchange in L2 to the thread that holds the mirror
-// (unit 2^S0 - lo, index KEEP_R-1-i; KEEP_R-i for lo = 0).  X[K] leaves by
-// TMA from the staged ranges, X[N-K] from the ranges staged in reverse
-// through omap2 (W x 256 boxes at any row; the one row past the image, the
-// mirror of K = 0, is outside the map and not written); X[N/2], which pairs
-// with itself, is stored by CTA 0's threads of row 0 (io.mid_row).
-template <class C, int CL, bool H16, int DCT = 0>
+template <class C, int CL, bool H16>
 __device__ __forceinline__ void col_group_l2_body(const CUtensorMap *lmap, const CUtensorMap *omap,
                                                   int ntiles, const float2 *__restrict__ tw,
                                                   float scale, int *err, int withhold,
-                                                  float2 *xbuf, const GroupIO &io,
-                                                  const CUtensorMap *lmap2 = nullptr,
-                                                  const float2 *__restrict__ post = nullptr,
-                                                  const CUtensorMap *omap2 = nullptr)
+                                                  float2 *xbuf, const GroupIO &io)
 {
     namespace cg = cooperative_groups;
     using S = TmaSplit<C>;
@@ -673,10 +612,6 @@ __device__ __forceinline__ void col_group_l2_body(const CUtensorMap *lmap, const
     __shared__ int lost_flag[2][CS];       // [tile parity][slot p: written by CTA p]
     __shared__ int cmax[2][CS][C::W];      // half2: [tile parity][CTA p's partial column maxima]
     __shared__ int cmax_local[C::W];
-    // DCT == 3: (cos, sin)(pi B / (2N)) of the block starts B = NL t + k_base
-    // + 2^S0 i of this CTA's paired outputs (t < CS/2); a thread multiplies
-    // them by its own (cos, sin)(pi lo / (2N)) (within a few ulp of the table)
-    __shared__ float2 rot_base[DCT == 3 ? (1 << CL) / 2 * (Grp<C, C::NG - 1>::R >> CL) : 1];
     cg::cluster_group cluster = cg::this_cluster();
     const int q = (int)cluster.block_rank();
     const int tid = threadIdx.x;
@@ -687,24 +622,9 @@ __device__ __forceinline__ void col_group_l2_body(const CUtensorMap *lmap, const
     float *rf = reinterpret_cast<float *>(smb + GH::RF_OFF);
     const uint32_t tw_bytes = H16 ? (uint32_t)C::N * 8u : S::TW_BYTES;
     float2 *stage = sm + C::E / 2;
-    static_assert(!(H16 && DCT), "one storage mode");
-    constexpr uint32_t DCT_HALF_BYTES = (uint32_t)(C::N / 2) * C::W * 4u;   // floats
-    constexpr int DCT_HALF_FLOATS = (C::N / 2) * C::W;
     // the first and second half of a tile's TMA boxes
     auto issue_early = [&](int t) {
-        if constexpr (DCT == 1) {
-            mbar_arrive_expect_tx(&bar_early, DCT_HALF_BYTES);
-            tma_load_3d(sm + C::E, lmap, t * (C::W / 2), 0, 0, &bar_early);
-        } else if constexpr (DCT == 3) {
-            mbar_arrive_expect_tx(&bar_early, S::EARLY_BYTES);
-            tma_load_3d(sm + C::E, lmap, t * C::W, 0, 0, &bar_early);
-        } else if constexpr (DCT == 2) {
-            // first halves of the natural and the mirrored rows
-            float *pf = reinterpret_cast<float *>(sm + C::E);
-            mbar_arrive_expect_tx(&bar_early, 2 * DCT_HALF_BYTES);
-            tma_load_3d(pf, lmap, t * (C::W / 2), 0, 0, &bar_early);
-            tma_load_3d(pf + DCT_HALF_FLOATS, lmap2, t * (C::W / 2), 0, 0, &bar_early);
-        } else if constexpr (H16) {
+        if constexpr (H16) {
             mbar_arrive_expect_tx(&bar_early, GH::HALF_BYTES);
             tma_load_3d(smb + GH::PREF_OFF, lmap, t * C::W, 0, 0, &bar_early);
         } else {
@@ -712,19 +632,7 @@ __device__ __forceinline__ void col_group_l2_body(const CUtensorMap *lmap, const
         }
     };
     auto issue_late = [&](int t) {
-        if constexpr (DCT == 1) {
-            mbar_arrive_expect_tx(&bar_late, DCT_HALF_BYTES);
-            tma_load_3d(sm, lmap2, t * (C::W / 2), 0, 0, &bar_late);
-        } else if constexpr (DCT == 3) {
-            mbar_arrive_expect_tx(&bar_late, S::LATE_BYTES);
-            tma_load_3d(sm, lmap2, t * C::W, 0, 0, &bar_late);
-        } else if constexpr (DCT == 2) {
-            // second halves, at the start of the tile region
-            float *lf = reinterpret_cast<float *>(sm);
-            mbar_arrive_expect_tx(&bar_late, 2 * DCT_HALF_BYTES);
-            tma_load_3d(lf, lmap, t * (C::W / 2), 0, S::NB, &bar_late);
-            tma_load_3d(lf + DCT_HALF_FLOATS, lmap2, t * (C::W / 2), 0, S::NB, &bar_late);
-        } else if constexpr (H16) {
+        if constexpr (H16) {
             mbar_arrive_expect_tx(&bar_late, GH::HALF_BYTES);
             tma_load_3d(smb, lmap, t * C::W, 0, GH::NB, &bar_late);
         } else {
@@ -736,7 +644,7 @@ __device__ __forceinline__ void col_group_l2_body(const CUtensorMap *lmap, const
     constexpr bool R4 = CL == 2;
     constexpr bool VEC = H16;   // 16-byte exchange slots (see group_round_send_g)
     constexpr int R4V = GC::KEEP_V;                       // values per source and destination
-    constexpr long long XSTRIDE = GC::L2_SCRATCH_VALS + (DCT == 3 ? GC::MIRROR_VALS : 0);
+    constexpr long long XSTRIDE = GC::L2_SCRATCH_VALS;
     float2 *xb = xbuf + (long long)cid * XSTRIDE + tid;
     int rk_end = 0;
 #pragma unroll
@@ -749,13 +657,6 @@ __device__ __forceinline__ void col_group_l2_body(const CUtensorMap *lmap, const
         mbar_init(&bar_early, 1);
         mbar_init(&bar_late, 1);
         fence_mbar_init();
-    }
-    float2 rot_lo = make_float2(1.f, 0.f);
-    if constexpr (DCT == 3) {
-        constexpr int KR = GC::KEEP_R;
-        for (int j = tid; j < CS / 2 * KR; j += C::T)
-            rot_base[j] = __ldg(post + ((j / KR) << C::L) + k_base + ((j % KR) << Gl::S0));
-        rot_lo = __ldg(post + ((tid >> C::KW) & ((1 << Gl::S0) - 1)));
     }
     if constexpr (H16) {
         // the factors of this CTA's rows CS m + rev_CL(q)
@@ -796,131 +697,7 @@ __device__ __forceinline__ void col_group_l2_body(const CUtensorMap *lmap, const
         if (!lost_here) {
             w_early++;
             w_late++;
-            if constexpr (DCT == 2) {
-                // group 0: scrambled gather of the spectrum rows k = CS i +
-                // res and their mirrors N - k, pre-rotated into V[k]
-                const int res = brev_rt(q, CL);
-                constexpr int NN = C::N << CL;
-                const float *pn = reinterpret_cast<const float *>(sm + C::E);
-                const float *pm = pn + DCT_HALF_FLOATS;
-                const float *ln = reinterpret_cast<const float *>(sm);
-                const float *lm = ln + DCT_HALF_FLOATS;
-#pragma unroll
-                for (int v = 0; v < G0::V; v++) {
-                    const int u = tid + v * C::T;
-                    const int w = u & (C::W - 1);
-                    const int hib = (u >> C::KW) & ((1 << G0::HB) - 1);
-#pragma unroll
-                    for (int r = 0; r < G0::R; r++) {
-                        const int top = brev_c(r, G0::G) << G0::HB;   // compile-time
-                        const int i = top | hib;
-                        const float xn = top < C::N / 2 ? pn[i * C::W + w]
-                                                        : ln[(i - C::N / 2) * C::W + w];
-                        const int j = res == 0 ? ((C::N - i) & (C::N - 1)) : C::N - 1 - i;
-                        float xm = j < C::N / 2 ? pm[j * C::W + w] : lm[(j - C::N / 2) * C::W + w];
-                        if (res == 0 && i == 0)
-                            xm = 0.f;   // X[N] = 0
-                        const int k = CS * i + res;
-                        const float2 cs = k <= NN / 2 ? __ldg(post + k) : __ldg(post + (NN - k));
-                        const float c = k <= NN / 2 ? cs.x : cs.y;
-                        const float sn = k <= NN / 2 ? cs.y : cs.x;
-                        a[v * G0::R + r] = make_float2(c * xn + sn * xm, sn * xn - c * xm);
-                    }
-                }
-#pragma unroll
-                for (int v = 0; v < G0::V; v++)
-                    run_stages<C, 0, false, true>(a, v, 0, stw, C::L);
-                fence_proxy_async_smem();
-                if (tid == 0)
-                    bulk_wait_read_all();   // the previous tile's stores have read it
-                __syncthreads();            // every slot of both input regions has been read
-                if (tid == 0 && next < ntiles)
-                    issue_early(next);
-#pragma unroll
-                for (int v = 0; v < G0::V; v++) {
-                    const int u = tid + v * C::T;
-                    const int w = u & (C::W - 1);
-                    const int hib = (u >> C::KW) & ((1 << G0::HB) - 1);
-                    const int hi = brev_rt(hib, G0::HB);
-#pragma unroll
-                    for (int r = 0; r < G0::R; r++)
-                        sm[sidx<C>(0, r | (hi << G0::G), w)] = a[v * G0::R + r];
-                }
-            } else if constexpr (DCT == 3) {
-                // group 0: scrambled gather of the reordered pairs of real
-                // columns (the second half of the local line read backwards)
-                const float2 *pref = sm + C::E;
-                const float2 *late = sm;
-#pragma unroll
-                for (int v = 0; v < G0::V; v++) {
-                    const int u = tid + v * C::T;
-                    const int w = u & (C::W - 1);
-                    const int hib = (u >> C::KW) & ((1 << G0::HB) - 1);
-#pragma unroll
-                    for (int r = 0; r < G0::R; r++) {
-                        const int top = brev_c(r, G0::G) << G0::HB;   // compile-time
-                        a[v * G0::R + r] = top < C::N / 2 ? pref[(top | hib) * C::W + w]
-                                                          : late[(C::N - 1 - (top | hib)) * C::W + w];
-                    }
-                }
-#pragma unroll
-                for (int v = 0; v < G0::V; v++)
-                    run_stages<C, 0, false, true>(a, v, 0, stw, C::L);
-                fence_proxy_async_smem();
-                if (tid == 0)
-                    bulk_wait_read_all();   // the previous tile's stores have read it
-                __syncthreads();            // every slot of both input regions has been read
-                if (tid == 0 && next < ntiles)
-                    issue_early(next);
-#pragma unroll
-                for (int v = 0; v < G0::V; v++) {
-                    const int u = tid + v * C::T;
-                    const int w = u & (C::W - 1);
-                    const int hib = (u >> C::KW) & ((1 << G0::HB) - 1);
-                    const int hi = brev_rt(hib, G0::HB);
-#pragma unroll
-                    for (int r = 0; r < G0::R; r++)
-                        sm[sidx<C>(0, r | (hi << G0::G), w)] = a[v * G0::R + r];
-                }
-            } else if constexpr (DCT == 1) {
-                // group 0: scrambled gather of the reordered real columns
-                // (the second half of the local line read backwards), as
-                // complex values with imaginary part zero
-                const float *pref = reinterpret_cast<const float *>(sm + C::E);
-                const float *late = reinterpret_cast<const float *>(sm);
-#pragma unroll
-                for (int v = 0; v < G0::V; v++) {
-                    const int u = tid + v * C::T;
-                    const int w = u & (C::W - 1);
-                    const int hib = (u >> C::KW) & ((1 << G0::HB) - 1);
-#pragma unroll
-                    for (int r = 0; r < G0::R; r++) {
-                        const int top = brev_c(r, G0::G) << G0::HB;   // compile-time
-                        const float x = top < C::N / 2 ? pref[(top | hib) * C::W + w]
-                                                       : late[(C::N - 1 - (top | hib)) * C::W + w];
-                        a[v * G0::R + r] = make_float2(x, 0.f);
-                    }
-                }
-#pragma unroll
-                for (int v = 0; v < G0::V; v++)
-                    run_stages<C, 0, false, true>(a, v, 0, stw, C::L);
-                fence_proxy_async_smem();
-                if (tid == 0)
-                    bulk_wait_read_all();   // the previous tile's stores have read it
-                __syncthreads();            // every slot of both input regions has been read
-                if (tid == 0 && next < ntiles)
-                    issue_early(next);
-#pragma unroll
-                for (int v = 0; v < G0::V; v++) {
-                    const int u = tid + v * C::T;
-                    const int w = u & (C::W - 1);
-                    const int hib = (u >> C::KW) & ((1 << G0::HB) - 1);
-                    const int hi = brev_rt(hib, G0::HB);
-#pragma unroll
-                    for (int r = 0; r < G0::R; r++)
-                        sm[sidx<C>(0, r | (hi << G0::G), w)] = a[v * G0::R + r];
-                }
-            } else if constexpr (H16) {
+            if constexpr (H16) {
                 // group 0: scrambled gather of the half2 tile, widened and
                 // scaled by the row factors
                 const __half2 *pref = reinterpret_cast<const __half2 *>(smb + GH::PREF_OFF);
@@ -1121,189 +898,6 @@ __device__ __forceinline__ void col_group_l2_body(const CUtensorMap *lmap, const
             const float2 *theirs = x0 + (q ^ 1) * XV;
             group_round_compute_g<C, 0, VEC>(a, theirs, wk, q & 1);
         }
-        if constexpr (DCT == 3) {
-            constexpr int NN = C::N << CL;   // line length
-            constexpr int HT = CS / 2;       // blocks t < HT are paired here
-            constexpr int KR = GC::KEEP_R;
-            constexpr int MREG = HT * GC::KEEP_V * C::T;
-            static_assert(Gl::V == 1 && C::T == (1 << (Gl::S0 + C::KW)), "one unit per thread");
-            float2 *mb = xbuf + (long long)cid * XSTRIDE + GC::L2_SCRATCH_VALS;
-            const int w = tid & (C::W - 1);
-            const int lo = tid >> C::KW;
-            {
-                // blocks t >= HT to CTA CS-1-q, each value in the slot of
-                // the thread and index that pair it
-                float2 *dst = mb + (CS - 1 - q) * MREG;
-                const int tid_r = ((((1 << Gl::S0) - lo) & ((1 << Gl::S0) - 1)) << C::KW) | w;
-#pragma unroll
-                for (int t = HT; t < CS; t++) {
-#pragma unroll
-                    for (int i = 0; i < KR; i++) {
-                        if (lo == 0 && i == 0)
-                            continue;
-                        const int i_r = lo != 0 ? KR - 1 - i : KR - i;
-                        __stcg(dst + ((CS - 1 - t) * KR + i_r) * C::T + tid_r, a[t * KR + i]);
-                    }
-                }
-                // row 0 of CTAs 2 and 3 of four: the other one pairs it
-                if (CL == 2 && q >= 2 && lo == 0) {
-                    float2 *d2 = mb + (q ^ 1) * MREG;
-#pragma unroll
-                    for (int t = HT; t < CS; t++)
-                        __stcg(d2 + (CS - 1 - t) * KR * C::T + w, a[t * KR]);
-                }
-            }
-            cluster_arrive_release();   // the mirror values are visible
-            float2 r0[CS];              // row 0 of every block
-#pragma unroll
-            for (int t = 0; t < CS; t++)
-                r0[t] = a[t * KR];
-            if (q == 0 && lo == 0) {
-                // K = N/2: row 0 of block HT in CTA 0, its own mirror
-                float2 xk, xp;
-                dct_pair(r0[HT], r0[HT], __ldg(post + NN / 2), scale, xk, xp);
-                st_stream(io.mid_row + (long long)tile * C::W + w, xk);
-            }
-            cluster_wait_acquire();
-            const float2 *src = mb + q * MREG + tid;
-#pragma unroll
-            for (int t = 0; t < HT; t++) {
-#pragma unroll
-                for (int i = 0; i < KR; i++) {
-                    const float2 zk = a[t * KR + i];
-                    float2 zp;
-                    if (i == 0 && lo == 0 && q == 0)
-                        zp = t == 0 ? zk : r0[CS - t];   // K = 0 and NL t: CTA 0's own
-                    else if (i == 0 && lo == 0 && k_base == C::N / 2)
-                        zp = r0[CS - 1 - t];             // k = NL/2 mirrors itself
-                    else
-                        zp = __ldcg(src + (t * KR + i) * C::T);
-                    const float2 rb = rot_base[t * KR + i];
-                    const float2 cs = make_float2(rb.x * rot_lo.x - rb.y * rot_lo.y,
-                                                  rb.x * rot_lo.y + rb.y * rot_lo.x);
-                    float2 xk, xp;
-                    dct_pair(zk, zp, cs, scale, xk, xp);
-                    a[t * KR + i] = xk;
-                    a[(t + HT) * KR + i] = xp;
-                }
-            }
-            // X[K] of blocks t < HT: one staging fill, one TMA store per range
-#pragma unroll
-            for (int t = 0; t < HT; t++)
-#pragma unroll
-                for (int i = 0; i < KR; i++)
-                    stage[(t * GC::OUT_ROWS + ((i << Gl::S0) | lo)) * C::W + w] = a[t * KR + i];
-            fence_proxy_async_smem();
-            __syncthreads();
-            if (tid == 0) {
-#pragma unroll
-                for (int t = 0; t < HT; t++)
-                    tma_store_3d(omap, tile * C::W, 0, ((t << C::L) + k_base) / S::BOX,
-                                 stage + t * GC::OUT_ROWS * C::W);
-                bulk_commit();
-                bulk_wait_read_all();
-            }
-            __syncthreads();
-            // X[N-K]: the same ranges in reverse, rows y0 + s, y0 = N - NL t
-            // - k_base - OUT_ROWS + 1, in 256-row boxes of omap2
-#pragma unroll
-            for (int t = 0; t < HT; t++)
-#pragma unroll
-                for (int i = 0; i < KR; i++)
-                    stage[(t * GC::OUT_ROWS + GC::OUT_ROWS - 1 - ((i << Gl::S0) | lo)) * C::W + w] =
-                        a[(t + HT) * KR + i];
-            fence_proxy_async_smem();
-            __syncthreads();
-            if (tid == 0) {
-#pragma unroll
-                for (int t = 0; t < HT; t++) {
-                    const int y0 = NN - (t << C::L) - k_base - GC::OUT_ROWS + 1;
-#pragma unroll
-                    for (int j = 0; j < GC::OUT_BOX_Z; j++)
-                        tma_store_3d(omap2, tile * C::W, y0 + j * S::BOX, 0,
-                                     stage + (t * GC::OUT_ROWS + j * S::BOX) * C::W);
-                }
-                bulk_commit();
-            }
-            continue;
-        }
-        if constexpr (DCT == 2) {
-            // x[2n] = Re v[n] (n < N/2, the even rows), x[2(N-1-n)+1] = Re
-            // v[n] (the odd rows, in reverse order within a range)
-            float *fst = reinterpret_cast<float *>(stage);
-#pragma unroll
-            for (int t = 0; t < CS; t++) {
-                const bool odd = t >= CS / 2;
-#pragma unroll
-                for (int v = 0; v < Gl::V; v++) {
-                    const int u = tid + v * C::T;
-                    const int w = u & (C::W - 1);
-                    const int lo = (u >> C::KW) & ((1 << Gl::S0) - 1);
-#pragma unroll
-                    for (int i = 0; i < GC::KEEP_R; i++) {
-                        const int row = (i << Gl::S0) | lo;
-                        const int slot = odd ? GC::OUT_ROWS - 1 - row : row;
-                        fst[(t * GC::OUT_ROWS + slot) * C::W + w] =
-                            a[(t * Gl::V + v) * GC::KEEP_R + i].x * scale;
-                    }
-                }
-            }
-            fence_proxy_async_smem();
-            __syncthreads();
-            if (tid == 0) {
-                constexpr int NN = C::N << CL;
-#pragma unroll
-                for (int t = 0; t < CS; t++) {
-                    const int n0 = (t << C::L) + k_base;
-                    if (t < CS / 2)
-                        tma_store_3d(omap, tile * (C::W / 2), 0, n0 / S::BOX,
-                                     fst + t * GC::OUT_ROWS * C::W);
-                    else
-                        tma_store_3d(omap2, tile * (C::W / 2), 0,
-                                     (NN - n0 - GC::OUT_ROWS) / S::BOX,
-                                     fst + t * GC::OUT_ROWS * C::W);
-                }
-                bulk_commit();
-            }
-            continue;
-        }
-        if constexpr (DCT == 1) {
-            // X[K] = cos(theta) Re V[K] + sin(theta) Im V[K], theta = pi K /
-            // (2N), K = k + 2^L t; (cos, sin) of K > N/2 is (sin, cos) of N - K
-            constexpr int NN = C::N << CL;
-            float *fst = reinterpret_cast<float *>(stage);
-#pragma unroll
-            for (int t = 0; t < CS; t++) {
-#pragma unroll
-                for (int v = 0; v < Gl::V; v++) {
-                    const int u = tid + v * C::T;
-                    const int w = u & (C::W - 1);
-                    const int lo = (u >> C::KW) & ((1 << Gl::S0) - 1);
-#pragma unroll
-                    for (int i = 0; i < GC::KEEP_R; i++) {
-                        const int row = (i << Gl::S0) | lo;
-                        const int K = (t << C::L) + k_base + row;
-                        const float2 cs = K <= NN / 2 ? __ldg(post + K) : __ldg(post + (NN - K));
-                        const float c = K <= NN / 2 ? cs.x : cs.y;
-                        const float sn = K <= NN / 2 ? cs.y : cs.x;
-                        const float2 z = a[(t * Gl::V + v) * GC::KEEP_R + i];
-                        fst[(t * GC::OUT_ROWS + row) * C::W + w] = (c * z.x + sn * z.y) * scale;
-                    }
-                }
-            }
-            fence_proxy_async_smem();
-            __syncthreads();
-            if (tid == 0) {
-#pragma unroll
-                for (int t = 0; t < CS; t++) {
-                    const int z = ((t << C::L) + k_base) / S::BOX;
-                    tma_store_3d(omap, tile * (C::W / 2), 0, z,
-                                 fst + t * GC::OUT_ROWS * C::W);
-                }
-                bulk_commit();
-            }
-            continue;
-        }
         if constexpr (H16) {
             // this CTA's part of each column's largest |component| (a
             // thread's values all belong to column tid mod W) to every CTA of
@@ -1412,74 +1006,6 @@ __device__ __forceinline__ void col_group_l2_body(const CUtensorMap *lmap, const
     }
     if (tid == 0)
         bulk_wait_all();   // shared memory stays valid until the stores are done
-}
-
-// The forward DCT-II column pass of real columns on the same kernel (DCT
-// mode above): per residue rev(q) a map of the ascending rows (first half of
-// the local line) and one of the rows read backwards (second half).
-struct DctL2Maps {
-    CUtensorMap early[4], late[4];
-    CUtensorMap out;
-};
-
-template <class C, int CL>
-__global__ void __launch_bounds__(C::T, 1) col_dct_l2_kernel(const __grid_constant__ DctL2Maps maps,
-                                                             const float2 *__restrict__ tw,
-                                                             const float2 *__restrict__ post,
-                                                             int ntiles, float scale, int *err,
-                                                             int withhold, float2 *xbuf)
-{
-    const int q = (int)cooperative_groups::this_cluster().block_rank();
-    const int res = brev_rt(q, CL);
-    col_group_l2_body<C, CL, false, 1>(&maps.early[res], &maps.out, ntiles, tw, scale, err,
-                                       withhold, xbuf, GroupIO{nullptr, nullptr}, &maps.late[res],
-                                       post);
-}
-
-// The forward DCT-II column pass with two real columns per complex line
-// (DCT == 3 above): per residue the complex maps of the ascending and the
-// backwards rows, the output map of whole ranges, the any-row map of the
-// reversed ranges, and the output row N/2.
-struct DctPackMaps {
-    CUtensorMap early[4], late[4];
-    CUtensorMap out, out2;
-    float2 *mid_row;
-};
-
-template <class C, int CL>
-__global__ void __launch_bounds__(C::T, 1) col_dct_pack_l2_kernel(
-    const __grid_constant__ DctPackMaps maps, const float2 *__restrict__ tw,
-    const float2 *__restrict__ post, int ntiles, float scale, int *err, int withhold,
-    float2 *xbuf)
-{
-    const int q = (int)cooperative_groups::this_cluster().block_rank();
-    const int res = brev_rt(q, CL);
-    col_group_l2_body<C, CL, false, 3>(&maps.early[res], &maps.out, ntiles, tw, scale, err,
-                                       withhold, xbuf, GroupIO{nullptr, nullptr, maps.mid_row},
-                                       &maps.late[res], post, &maps.out2);
-}
-
-// The inverse DCT-III column pass of real columns (DCT == 2 above): per
-// residue a map of its rows (the mirror of residue r is residue (CS-r) mod
-// CS), and store maps over the even and the odd rows of the output.
-struct IdctL2Maps {
-    CUtensorMap rows[4];
-    CUtensorMap even, odd;
-};
-
-template <class C, int CL>
-__global__ void __launch_bounds__(C::T, 1) col_idct_l2_kernel(const __grid_constant__ IdctL2Maps maps,
-                                                              const float2 *__restrict__ tw,
-                                                              const float2 *__restrict__ post,
-                                                              int ntiles, float scale, int *err,
-                                                              int withhold, float2 *xbuf)
-{
-    constexpr int CS = 1 << CL;
-    const int q = (int)cooperative_groups::this_cluster().block_rank();
-    const int res = brev_rt(q, CL);
-    col_group_l2_body<C, CL, false, 2>(&maps.rows[res], &maps.even, ntiles, tw, scale, err,
-                                       withhold, xbuf, GroupIO{nullptr, nullptr},
-                                       &maps.rows[(CS - res) & (CS - 1)], post, &maps.odd);
 }
 
 template <class C, int CL, bool H16 = false>

@@ -34,12 +34,11 @@
 //    passes for columns of 2^11 points;
 //  * col_dct_tma64_kernel / col_idct_tma64_kernel: columns of 2^12 points on
 //    the 6-stage engine of the complex column pass;
-//  * col_dct_pack_l2_kernel (col_group.cuh): forward columns of 2^13 and
-//    2^14 points on a cluster of 2 or 4 CTAs, two real columns per complex
-//    line; col_idct_pair_kernel and col_idct_l2_kernel: the inverse.
+//  * col_strip.cu: columns of 2^13 and 2^14 points, in two phases through a
+//    scratch strip in L2.
 #include <cmath>
 
-#include "col_group.cuh"
+#include "dct_math.cuh"
 #include "line_fft.cuh"
 #include "passes.h"
 
@@ -75,7 +74,7 @@ __device__ __forceinline__ float2 dct_load(const DctIO &d, long long line0, int 
     }
 }
 
-// dct_pair (col_group.cuh): the outputs at k and k' = (N - k) mod N of
+// dct_pair (dct_math.cuh): the outputs at k and k' = (N - k) mod N of
 // the two real lines of a complex line, from Z[k] and Z[k'].
 
 template <class C, bool ROW>
@@ -243,14 +242,6 @@ __global__ void __launch_bounds__(C::T, C::MINB) line_dct_kernel(const DctIO d,
 //   Z[k]   = (c + i s) ((X_a[k] + X_b[N-k]) + i (X_b[k] - X_a[N-k])),
 //   Z[N-k] = (s + i c) ((X_a[N-k] + X_b[k]) + i (X_b[N-k] - X_a[k])),
 // (c, s) = (cos, sin)(pi k / (2N)); Z[0] = z[0].
-__device__ __forceinline__ void idct_pre(float2 za, float2 zb, float2 cs, float2 &yk, float2 &yp)
-{
-    const float ux = za.x + zb.y, uy = za.y - zb.x;
-    const float vx = zb.x + za.y, vy = zb.y - za.x;
-    yk = make_float2(cs.x * ux - cs.y * uy, cs.y * ux + cs.x * uy);
-    yp = make_float2(cs.y * vx - cs.x * vy, cs.x * vx + cs.y * vy);
-}
-
 // The un-reordering store of v[n] and v[N-1-n] (n < N/2) of complex line lb
 // (rows: real rows 2(line0+lb), +1; columns: complex column line0 + w).
 template <bool ROW>
@@ -1335,247 +1326,6 @@ cudaError_t idct_col_tma64_launch(const DctIO &d, const float2 *tw, const float2
     return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, oe, oo, ntiles, tw, post, scale, err, withhold);
 }
 
-// ---------------------------------------------------------------------------
-// Tile geometry of the inverse DCT column pass over a CTA pair (below): the
-// local engine's 2^L rows in two halves of whole 256-row blocks.
-template <class C>
-struct DctPair {
-    using S = TmaSplit<C>;
-    using GC = GroupCol<C, 1>;
-    static constexpr int HALF_ROWS = C::N / 2;               // local rows per map
-    static constexpr uint32_t HBYTES = (uint32_t)HALF_ROWS * C::W * 8u;
-    static constexpr int NBH = HALF_ROWS / S::BOX;           // 256-row blocks per map
-    static_assert(C::L == 12 && C::W == 4, "the 4096-row engine, 4 complex columns");
-    static_assert(HBYTES == S::EARLY_BYTES && HBYTES == S::LATE_BYTES, "two halves of the split");
-};
-
-// Forward DCT columns of 16384 points on the four-CTA cluster kernel with
-// the exchange through L2 (col_dct_l2_kernel, one complex line per real
-// column), for widths of 4 mod 8 real columns (the packed kernel above takes
-// multiples of 8); cudaErrorNotSupported (nothing launched) when the image
-// does not allow it.  The kernel runs in place: its tiles are 4 real columns, so
-// every access is half of a 32-byte sector, and a store merges into a
-// sector that the load of the same tile (and of the neighbouring tile, in
-// flight at the same time) has just brought into L2.  Out of place the
-// stores would fall on sectors not in L2 (measured 3.38 ms against 1.35 ms
-// at 16384^2, with 25 % more DRAM reads), so an out-of-place call copies the
-// input to the output first (one device-to-device copy).
-cudaError_t dct_col_quad_launch(const DctIO &din, const float2 *tw, const float2 *post,
-                                float scale, int *err, int withhold, cudaStream_t s)
-{
-    using C = LineCfg<12, 2, 0, 64, 6>;
-    using S = TmaSplit<C>;
-    using GC = GroupCol<C, 2>;
-    constexpr int CS = GC::CS;
-    const long long cc = din.cols / 2;   // 8-byte elements per row
-    if (!err || din.rows != (long long)CS * C::N || din.cols % C::W != 0 ||
-        (reinterpret_cast<uintptr_t>(din.in) & 15) || (reinterpret_cast<uintptr_t>(din.out) & 15) ||
-        (reinterpret_cast<uintptr_t>(tw) & 15) || !tensor_maps_available())
-        return cudaErrorNotSupported;
-    const DctIO d{din.out, din.out, din.rows, din.cols};
-    const float2 *in = reinterpret_cast<const float2 *>(d.in);
-    float2 *out = reinterpret_cast<float2 *>(d.out);
-    constexpr int HALF = C::N / 2;   // rows of each half of a CTA's local line
-    DctL2Maps m;
-    for (int r = 0; r < CS; r++)
-        if (!encode_col_map(&m.early[r], in + 2 * r * cc, HALF, (int)cc, 2 * CS * cc, C::W / 2,
-                            S::BOX, HALF / S::BOX) ||
-            !encode_col_map(&m.late[r], in + (2 * CS - 1 - 2 * r) * cc, HALF, (int)cc, 2 * CS * cc,
-                            C::W / 2, S::BOX, HALF / S::BOX))
-            return cudaErrorNotSupported;
-    if (!encode_col_map(&m.out, out, (int)d.rows, (int)cc, cc, C::W / 2, S::BOX, GC::OUT_BOX_Z))
-        return cudaErrorNotSupported;
-    auto k = col_dct_l2_kernel<C, 2>;
-    constexpr int SMEM = S::SMEM_BYTES;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(C::T);
-    cfg.dynamicSmemBytes = SMEM;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    static DeviceCache groups;
-    const int dev = device_current();
-    if (!groups.get(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e != cudaSuccess)
-            return e;
-        cfg.gridDim = dim3((unsigned)(CS * (device_sm_count() / CS)));
-        int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
-        if (e != cudaSuccess)
-            return e;
-        groups.set(dev, n > 0 ? n : 1);
-    }
-    const int ntiles = (int)(d.cols / C::W);
-    const int ng = groups.get(dev) < ntiles ? groups.get(dev) : ntiles;
-    if (din.in != din.out) {
-        cudaError_t e = cudaMemcpyAsync(din.out, din.in, (size_t)(din.rows * din.cols) * sizeof(float),
-                                        cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess)
-            return e;
-    }
-    void *xbuf = nullptr;
-    cudaError_t e = scratch_take(&xbuf, (size_t)ng * GC::L2_SCRATCH_VALS * sizeof(float2), s);
-    if (e != cudaSuccess)
-        return e;
-    cfg.gridDim = dim3((unsigned)(CS * ng));
-    e = cudaLaunchKernelEx(&cfg, k, m, tw, post, ntiles, scale, err, withhold,
-                           static_cast<float2 *>(xbuf));
-    const cudaError_t f = cudaFreeAsync(xbuf, s);
-    return e != cudaSuccess ? e : f;
-}
-
-// Forward DCT columns of 2^(12+CL) points (8192: a CTA pair, 16384: four
-// CTAs) with two real columns per complex line on the cluster kernel with
-// the exchange through L2 (col_dct_pack_l2_kernel): tiles of 8 real
-// columns, 32-byte rows, in place or out of place; cudaErrorNotSupported
-// (nothing launched) when the image does not allow it.
-template <int CL>
-cudaError_t dct_col_pack_launch(const DctIO &d, const float2 *tw, const float2 *post,
-                                float scale, int *err, int withhold, cudaStream_t s)
-{
-    using C = LineCfg<12, 2, 0, 64, 6>;
-    using S = TmaSplit<C>;
-    using GC = GroupCol<C, CL>;
-    constexpr int CS = GC::CS;
-    const long long cc = d.cols / 2;   // complex columns: pairs of real columns
-    if (!err || d.rows != (long long)CS * C::N || d.cols % (2 * C::W) != 0 ||
-        (reinterpret_cast<uintptr_t>(d.in) & 15) || (reinterpret_cast<uintptr_t>(d.out) & 15) ||
-        (reinterpret_cast<uintptr_t>(tw) & 15) || !tensor_maps_available())
-        return cudaErrorNotSupported;
-    const float2 *in = reinterpret_cast<const float2 *>(d.in);
-    float2 *out = reinterpret_cast<float2 *>(d.out);
-    constexpr int HALF = C::N / 2;   // rows of each half of a CTA's local line
-    DctPackMaps m;
-    for (int r = 0; r < CS; r++)
-        if (!encode_col_map(&m.early[r], in + 2 * r * cc, HALF, (int)cc, 2 * CS * cc, C::W, S::BOX,
-                            HALF / S::BOX) ||
-            !encode_col_map(&m.late[r], in + (2 * CS - 1 - 2 * r) * cc, HALF, (int)cc, 2 * CS * cc,
-                            C::W, S::BOX, HALF / S::BOX))
-            return cudaErrorNotSupported;
-    if (!encode_col_map(&m.out, out, (int)d.rows, (int)cc, cc, C::W, S::BOX, GC::OUT_BOX_Z) ||
-        !encode_map_xyz(&m.out2, out, cc, (int)d.rows, 1, cc, cc * d.rows, C::W, S::BOX, 1))
-        return cudaErrorNotSupported;
-    m.mid_row = out + (d.rows / 2) * cc;
-    auto k = col_dct_pack_l2_kernel<C, CL>;
-    constexpr int SMEM = S::SMEM_BYTES;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(C::T);
-    cfg.dynamicSmemBytes = SMEM;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    static DeviceCache groups;
-    const int dev = device_current();
-    if (!groups.get(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e != cudaSuccess)
-            return e;
-        cfg.gridDim = dim3((unsigned)(CS * (device_sm_count() / CS)));
-        int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
-        if (e != cudaSuccess)
-            return e;
-        groups.set(dev, n > 0 ? n : 1);
-    }
-    const int ntiles = (int)(cc / C::W);
-    const int ng = groups.get(dev) < ntiles ? groups.get(dev) : ntiles;
-    void *xbuf = nullptr;
-    cudaError_t e = scratch_take(
-        &xbuf, (size_t)ng * (size_t)(GC::L2_SCRATCH_VALS + GC::MIRROR_VALS) * sizeof(float2), s);
-    if (e != cudaSuccess)
-        return e;
-    cfg.gridDim = dim3((unsigned)(CS * ng));
-    e = cudaLaunchKernelEx(&cfg, k, m, tw, post, ntiles, scale, err, withhold,
-                           static_cast<float2 *>(xbuf));
-    const cudaError_t f = cudaFreeAsync(xbuf, s);
-    return e != cudaSuccess ? e : f;
-}
-
-// Inverse DCT columns of 16384 points on the same four-CTA kernel
-// (col_idct_l2_kernel, one real line per complex line), in place for the
-// same reason as the forward pass; cudaErrorNotSupported (nothing launched)
-// when the image does not allow it.
-cudaError_t idct_col_quad_launch(const DctIO &din, const float2 *tw, const float2 *post,
-                                 float scale, int *err, int withhold, cudaStream_t s)
-{
-    using C = LineCfg<12, 2, 0, 64, 6>;
-    using S = TmaSplit<C>;
-    using GC = GroupCol<C, 2>;
-    constexpr int CS = GC::CS;
-    const long long cc = din.cols / 2;   // 8-byte elements per row
-    if (!err || din.rows != (long long)CS * C::N || din.cols % C::W != 0 ||
-        (reinterpret_cast<uintptr_t>(din.in) & 15) || (reinterpret_cast<uintptr_t>(din.out) & 15) ||
-        (reinterpret_cast<uintptr_t>(tw) & 15) || !tensor_maps_available())
-        return cudaErrorNotSupported;
-    const DctIO d{din.out, din.out, din.rows, din.cols};
-    const float2 *in = reinterpret_cast<const float2 *>(d.in);
-    float2 *out = reinterpret_cast<float2 *>(d.out);
-    IdctL2Maps m;
-    for (int r = 0; r < CS; r++)
-        if (!encode_col_map(&m.rows[r], in + r * cc, C::N, (int)cc, CS * cc, C::W / 2, S::BOX,
-                            S::NB))
-            return cudaErrorNotSupported;
-    if (!encode_col_map(&m.even, out, (int)(d.rows / 2), (int)cc, 2 * cc, C::W / 2, S::BOX,
-                        GC::OUT_BOX_Z) ||
-        !encode_col_map(&m.odd, out + cc, (int)(d.rows / 2), (int)cc, 2 * cc, C::W / 2, S::BOX,
-                        GC::OUT_BOX_Z))
-        return cudaErrorNotSupported;
-    auto k = col_idct_l2_kernel<C, 2>;
-    constexpr int SMEM = S::SMEM_BYTES;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(C::T);
-    cfg.dynamicSmemBytes = SMEM;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    static DeviceCache groups;
-    const int dev = device_current();
-    if (!groups.get(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e != cudaSuccess)
-            return e;
-        cfg.gridDim = dim3((unsigned)(CS * (device_sm_count() / CS)));
-        int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
-        if (e != cudaSuccess)
-            return e;
-        groups.set(dev, n > 0 ? n : 1);
-    }
-    const int ntiles = (int)(d.cols / C::W);
-    const int ng = groups.get(dev) < ntiles ? groups.get(dev) : ntiles;
-    if (din.in != din.out) {
-        cudaError_t e = cudaMemcpyAsync(din.out, din.in, (size_t)(din.rows * din.cols) * sizeof(float),
-                                        cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess)
-            return e;
-    }
-    void *xbuf = nullptr;
-    cudaError_t e = scratch_take(&xbuf, (size_t)ng * GC::L2_SCRATCH_VALS * sizeof(float2), s);
-    if (e != cudaSuccess)
-        return e;
-    cfg.gridDim = dim3((unsigned)(CS * ng));
-    e = cudaLaunchKernelEx(&cfg, k, m, tw, post, ntiles, scale, err, withhold,
-                           static_cast<float2 *>(xbuf));
-    const cudaError_t f = cudaFreeAsync(xbuf, s);
-    return e != cudaSuccess ? e : f;
-}
-
 template <class C, bool ROW>
 cudaError_t dct_launch(const DctIO &d, const float2 *tw, const float2 *post, long long nlines,
                        float scale, cudaStream_t s)
@@ -1901,303 +1651,6 @@ __global__ void __launch_bounds__(C::T, 1) col_idct_tma_kernel(
         bulk_wait_all();
 }
 
-// ---------------------------------------------------------------------------
-// Inverse DCT column pass for columns of 2^(L+1) points over a CTA pair.
-// CTA b runs the DIT half of the inverse DFT whose inputs are the spectrum
-// positions k = 2m + b (the rows of parity b, one tensor map with twice the
-// row pitch).  The pre-rotation pairs k with N - k, which has the same
-// parity, so it stays inside the CTA: in local positions m pairs with
-// 2^L - m for b = 0 (m = 0 alone, m = 2^(L-1) with itself) and with
-// 2^L - 1 - m for b = 1.  A thread takes the group-0 units h and, for b = 0,
-// 2^HB - h (unit 0 with 2^(HB-1), both paired within themselves) or, for
-// b = 1, 2^HB - 1 - h.  After stages 1..L and the exchange round of stage
-// L+1, CTA b holds v[n] and v[n + 2^L] for n in [b 2^(L-1), (b+1) 2^(L-1));
-// x[2n] = v[n] and x[2n'+1] = v[N-1-n'] are two contiguous ranges of the
-// even and the odd output rows, each staged and stored with one TMA store.
-template <class C>
-__global__ void __launch_bounds__(C::T, 1) col_idct_pair_kernel(
-    const __grid_constant__ CUtensorMap m0, const __grid_constant__ CUtensorMap m1,
-    const __grid_constant__ CUtensorMap oe, const __grid_constant__ CUtensorMap oo, int ntiles,
-    const float2 *__restrict__ tw, const float2 *__restrict__ post, float scale, int *err,
-    int withhold)
-{
-    namespace cg = cooperative_groups;
-    using S = TmaSplit<C>;
-    using GC = GroupCol<C, 1>;
-    using G0 = Grp<C, 0>;
-    using Gl = Grp<C, C::NG - 1>;
-    constexpr int N = 2 * C::N;
-    constexpr int R = G0::R, HH = 1 << (G0::HB - 1);
-    static_assert(G0::V == 2 && (C::T >> C::KW) == HH, "threads cover half the group-0 units");
-    extern __shared__ __align__(1024) float2 sm[];
-    __shared__ __align__(8) uint64_t bar_early, bar_late, bar_recv;
-    __shared__ int lost_flag[2];
-    cg::cluster_group cluster = cg::this_cluster();
-    const int b = (int)cluster.block_rank();
-    const int tid = threadIdx.x;
-    pdl_wait();
-    const int nclusters = (int)gridDim.x / 2;
-    const CUtensorMap *lmap = b == 0 ? &m0 : &m1;
-    float2 *stw = sm + S::TW_OFF;
-    float2 *recvb = sm;
-    float2 *sendb = sm + C::E / 2;
-    const uint32_t peer_recv = mapa_shared(smem_addr(recvb), (uint32_t)(b ^ 1));
-    const uint32_t peer_bar = mapa_shared(smem_addr(&bar_recv), (uint32_t)(b ^ 1));
-    const int w = tid & (C::W - 1);
-    const int h = tid >> C::KW;
-    const int h1 = b == 0 ? (h == 0 ? HH : 2 * HH - h) : 2 * HH - 1 - h;
-    int lost_recv = 0;
-    int tile = (int)blockIdx.x / 2;
-    if (tid == 0) {
-        mbar_init(&bar_early, 1);
-        mbar_init(&bar_late, 1);
-        mbar_init(&bar_recv, 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-    int n_early = 0, n_late = 0, w_early = 0, w_late = 0;
-    if (tile < ntiles) {
-        if (tid == 0) {
-            mbar_expect_tx(&bar_early, S::TW_BYTES);
-            bulk_load(stw, tw, S::TW_BYTES, &bar_early);
-            split_issue_early<C>(sm, lmap, tile * C::W, &bar_early);
-            if (!(withhold && blockIdx.x == 0))   // self-test: the first late half never comes
-                split_issue_late<C>(sm, lmap, tile * C::W, &bar_late);
-        }
-        n_early = n_late = 1;
-    }
-    bool lost = false;
-    int w_recv = 0;
-    float2 a[C::EPT];
-    for (; tile < ntiles; tile += nclusters) {
-        const int next = tile + nclusters;
-        const bool ok = mbar_wait_bounded(&bar_early, (uint32_t)(w_early & 1)) &&
-                        mbar_wait_bounded(&bar_late, (uint32_t)(w_late & 1));
-        const int lost_here = __syncthreads_or((ok ? 0 : 1) | lost_recv);
-        if (tid == 0) {
-            if (!lost_recv)
-                mbar_arrive_expect_tx(&bar_recv, GC::XBYTES);
-            lost_flag[b] = lost_here;
-            *cluster.map_shared_rank(lost_flag + b, b ^ 1) = lost_here;
-        }
-        if (!lost_here) {
-            w_early++;
-            w_late++;
-#pragma unroll
-            for (int v = 0; v < 2; v++) {
-                const int hib = v ? h1 : h;
-#pragma unroll
-                for (int r = 0; r < R; r++) {
-                    const int top = brev_c(r, G0::G) << G0::HB;   // compile-time
-                    const int kb = top / S::BOX;
-                    const float2 *bx = kb < S::NB ? sm + C::E + kb * S::BOX_VALS
-                                                  : sm + (kb - S::NB) * S::BOX_VALS;
-                    a[v * R + r] = bx[((top % S::BOX) | hib) * C::W + w];
-                }
-            }
-            // pre-rotation of the pairs (k, N - k), k = 2 (local position) + b
-            float2 yk, yp;
-            if (b == 1 || h != 0) {
-#pragma unroll
-                for (int r = 0; r < R; r++) {
-                    const int rc = r ^ (R - 1);
-                    if (brev_c(r, G0::G) < R / 2) {
-                        const int ks = 2 * ((brev_c(r, G0::G) << G0::HB) + h) + b;
-                        idct_pre(a[r], a[R + rc], __ldg(post + ks), yk, yp);
-                        a[r] = yk;
-                        a[R + rc] = yp;
-                    } else {
-                        const int ks = 2 * ((brev_c(rc, G0::G) << G0::HB) + h1) + b;
-                        idct_pre(a[R + rc], a[r], __ldg(post + ks), yk, yp);
-                        a[R + rc] = yk;
-                        a[r] = yp;
-                    }
-                }
-            } else {
-                // b = 0, h = 0: unit 0 (positions brev(r) 2^HB) pairs b' with
-                // R - b' (k = 0 alone, k = N/2 with itself); unit HH pairs r
-                // with r ^ (R - 1)
-#pragma unroll
-                for (int bb = 1; bb < R / 2; bb++) {
-                    const int r = brev_c(bb, G0::G), r2 = brev_c(R - bb, G0::G);
-                    idct_pre(a[r], a[r2], __ldg(post + 2 * (bb << G0::HB)), yk, yp);
-                    a[r] = yk;
-                    a[r2] = yp;
-                }
-                constexpr int r8 = brev_c(R / 2, G0::G);
-                idct_pre(a[r8], a[r8], __ldg(post + N / 2), yk, yp);
-                a[r8] = yk;
-#pragma unroll
-                for (int r = 0; r < R; r++) {
-                    if (brev_c(r, G0::G) >= R / 2)
-                        continue;
-                    const int rc = r ^ (R - 1);
-                    idct_pre(a[R + r], a[R + rc],
-                             __ldg(post + 2 * ((brev_c(r, G0::G) << G0::HB) + HH)), yk, yp);
-                    a[R + r] = yk;
-                    a[R + rc] = yp;
-                }
-            }
-#pragma unroll
-            for (int v = 0; v < 2; v++)
-                run_stages<C, 0, false, true>(a, v, 0, stw, C::L);
-            fence_proxy_async_smem();
-            if (tid == 0)
-                bulk_wait_read_all();   // the previous tile's stores have read the staging
-            __syncthreads();
-            if (tid == 0 && next < ntiles)
-                split_issue_early<C>(sm, lmap, next * C::W, &bar_early);
-            if (next < ntiles)
-                n_early++;
-#pragma unroll
-            for (int v = 0; v < 2; v++) {
-                const int hi = brev_rt(v ? h1 : h, G0::HB);
-#pragma unroll
-                for (int r = 0; r < R; r++)
-                    sm[sidx<C>(0, r | (hi << G0::G), w)] = a[v * R + r];
-            }
-            __syncthreads();
-            group_smem<C, 1, false, false, true>(a, sm, stw, C::L);
-            __syncthreads();
-            group_last_read<C>(a, sm);
-            __syncthreads();   // the tile region is free
-        }
-        cluster_arrive_release();   // A0
-        float2 wk[16];
-        if (!lost_here) {
-#pragma unroll
-            for (int v = 0; v < Gl::V; v++) {
-                const int u = tid + v * C::T;
-                const int lo = (u >> C::KW) & ((1 << Gl::S0) - 1);
-                run_stages<C, C::NG - 1, false, true>(a, v, lo, stw, C::L);
-            }
-            group_round_send<C, 0>(a, sendb, b);
-            fence_proxy_async_smem();
-        }
-        __syncthreads();
-        group_round_twiddles<C, 0>(wk, tw, b * (Gl::R / 2));
-        cluster_wait_acquire();
-        if (lost_flag[0] | lost_flag[1]) {
-            lost = true;
-            break;
-        }
-        if (tid == 0)
-            bulk_copy_to_peer(peer_recv, sendb, GC::XBYTES, peer_bar);
-        lost_recv = mbar_wait_bounded(&bar_recv, (uint32_t)(w_recv & 1)) ? 0 : 1;
-        if (!lost_recv)
-            w_recv++;
-        cluster_arrive_release();   // B0: the partner's send buffer has been read
-        // stage L+1: a[t 16 + v 8 + i] = v[n + 2^L t], n = lo_v + 2^S0 (8b + i)
-        group_round_compute<C, 0>(a, recvb, wk, b);
-        fence_proxy_async_smem();
-        __syncthreads();   // the receive buffer has been read
-        if (tid == 0 && next < ntiles)
-            split_issue_late<C>(sm, lmap, next * C::W, &bar_late);
-        if (next < ntiles)
-            n_late++;
-        cluster_wait_acquire();   // B0: this CTA's send buffer is free for staging
-        // x[2n] = v[n]: even rows n in [b 2^(L-1), ...), one store; then
-        // x[2j+1] = v[N-1-j] = v[n + 2^L] for j = 2^L - 1 - n: odd rows
-        // j in [2^(L-1) (1 - b), ...), staged in reverse
-#pragma unroll
-        for (int t = 0; t < 2; t++) {
-            if (t == 1) {
-                if (tid == 0)
-                    bulk_wait_read_all();
-                __syncthreads();
-            }
-#pragma unroll
-            for (int v = 0; v < Gl::V; v++) {
-                const int lo = ((tid + v * C::T) >> C::KW) & ((1 << Gl::S0) - 1);
-#pragma unroll
-                for (int i = 0; i < 8; i++) {
-                    const int off = (i << Gl::S0) | lo;   // n - b 2^(L-1)
-                    const int slot = t == 0 ? off : (C::N / 2 - 1) - off;
-                    const float2 x = a[t * 16 + v * 8 + i];
-                    sendb[slot * C::W + w] = make_float2(x.x * scale, x.y * scale);
-                }
-            }
-            fence_proxy_async_smem();
-            __syncthreads();
-            if (tid == 0) {
-                if (t == 0)
-                    tma_store_3d(&oe, tile * C::W, 0, b * (C::N / 2 / S::BOX), sendb);
-                else
-                    tma_store_3d(&oo, tile * C::W, 0, (1 - b) * (C::N / 2 / S::BOX), sendb);
-                bulk_commit();
-            }
-        }
-    }
-
-    if (__syncthreads_or((lost || lost_recv) ? 1 : 0)) {
-        if (tid == 0)
-            atomicExch(err, kDevErrTmaTimeout);
-        if (n_early > w_early)
-            mbar_wait_bounded(&bar_early, (uint32_t)(w_early & 1));
-        if (n_late > w_late)
-            mbar_wait_bounded(&bar_late, (uint32_t)(w_late & 1));
-        if (lost_recv)
-            mbar_wait_bounded(&bar_recv, (uint32_t)(w_recv & 1));
-    }
-    if (tid == 0)
-        bulk_wait_all();
-}
-
-// The pair kernel for inverse DCT columns of 8192 points when the image
-// allows it; cudaErrorNotSupported otherwise.
-cudaError_t idct_col_pair_launch(const DctIO &d, const float2 *tw, const float2 *post,
-                                 float scale, int *err, int withhold, cudaStream_t s)
-{
-    using C = LineCfg<12, 2, 0, 32>;
-    using S = TmaSplit<C>;
-    using D = DctPair<C>;
-    const long long cc = d.cols / 2;
-    if (!err || d.rows != 2 * C::N || cc % C::W != 0 || (reinterpret_cast<uintptr_t>(d.in) & 15) ||
-        (reinterpret_cast<uintptr_t>(d.out) & 15) || (reinterpret_cast<uintptr_t>(tw) & 15) ||
-        (cc * 8) % 16 != 0 || !tensor_maps_available())
-        return cudaErrorNotSupported;
-    const float2 *in = reinterpret_cast<const float2 *>(d.in);
-    float2 *out = reinterpret_cast<float2 *>(d.out);
-    CUtensorMap lm[2], oe, oo;
-    for (int b = 0; b < 2; b++)
-        if (!encode_col_map(&lm[b], in + b * cc, C::N, (int)cc, 2 * cc, C::W, S::BOX, S::NB))
-            return cudaErrorNotSupported;
-    if (!encode_col_map(&oe, out, C::N, (int)cc, 2 * cc, C::W, S::BOX, D::NBH) ||
-        !encode_col_map(&oo, out + cc, C::N, (int)cc, 2 * cc, C::W, S::BOX, D::NBH))
-        return cudaErrorNotSupported;
-    auto k = col_idct_pair_kernel<C>;
-    constexpr int SMEM = S::SMEM_BYTES;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(C::T);
-    cfg.dynamicSmemBytes = SMEM;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    static DeviceCache pairs;
-    const int dev = device_current();
-    if (!pairs.get(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e != cudaSuccess)
-            return e;
-        cfg.gridDim = dim3((unsigned)(2 * (device_sm_count() / 2)));
-        int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
-        if (e != cudaSuccess)
-            return e;
-        pairs.set(dev, n > 0 ? n : 1);
-    }
-    const int ntiles = (int)(cc / C::W);
-    const int np = pairs.get(dev) < ntiles ? pairs.get(dev) : ntiles;
-    cfg.gridDim = dim3((unsigned)(2 * np));
-    return cudaLaunchKernelEx(&cfg, k, lm[0], lm[1], oe, oo, ntiles, tw, post, scale, err,
-                              withhold);
-}
-
 template <class C>
 cudaError_t idct_col_tma_launch(const DctIO &d, const float2 *tw, const float2 *post, float scale,
                                 int *err, int withhold, cudaStream_t s)
@@ -2232,6 +1685,14 @@ cudaError_t idct_col_tma_launch(const DctIO &d, const float2 *tw, const float2 *
     return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, oe, out, cc, ntiles, tw, post, dct_rot_table(), scale, err, withhold);
 }
 
+cudaError_t dct_col_strip(bool inverse, int L, const DctIO &d, const float2 *tw, const float2 *post,
+                          float scale, cudaStream_t s)
+{
+    const StripPass p{reinterpret_cast<const float2 *>(d.in), reinterpret_cast<float2 *>(d.out),
+                      d.cols / 2, (int)(d.cols / 2), tw, post, scale};
+    return launch_col_strip(inverse ? StripKind::Idct : StripKind::Dct, L, p, s);
+}
+
 template <int L>
 cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *tw,
                          const float2 *post, float scale, int *err, int withhold, cudaStream_t s)
@@ -2247,17 +1708,32 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
                                                                                 err, 1, s)
                            : dct_col_tma_launch<LineCfg<L, col_kw(L), 0, 32>>(d, tw, post, scale,
                                                                                err, 1, s);
-        if constexpr (L == 13)
-            return inverse ? idct_col_pair_launch(d, tw, post, scale, err, 1, s)
-                           : dct_col_pack_launch<1>(d, tw, post, scale, err, 1, s);
-        if constexpr (L == 14) {
-            if (inverse)
-                return idct_col_quad_launch(d, tw, post, scale, err, 1, s);
-            const cudaError_t e = dct_col_pack_launch<2>(d, tw, post, scale, err, 1, s);
-            return e != cudaErrorNotSupported ? e
-                                              : dct_col_quad_launch(d, tw, post, scale, err, 1, s);
+        // the strip passes of longer columns wait for nothing on the device:
+        // the TMA-fed complex64 pass of the same column length stands in
+        if constexpr (L >= 13) {
+            PassArgs a;
+            a.in = reinterpret_cast<const float2 *>(d.in);
+            a.out = reinterpret_cast<float2 *>(d.out);
+            a.tw = tw;
+            a.rows = (int)d.rows;
+            a.cols = (int)(d.cols / 2);
+            a.ld = d.cols / 2;
+            a.scale = scale;
+            a.nst = L;
+            a.partial = false;
+            a.err = err;
+            a.withhold = 1;
+            a.variant = col_selftest_variant(L, a);
+            return col_pass_is_tma_fed(L, a) ? launch_col_pass(L, a, s) : cudaErrorNotSupported;
         }
         return cudaErrorNotSupported;
+    }
+    if constexpr (L >= 13) {
+        if (!row) {
+            const cudaError_t e = dct_col_strip(inverse, L, d, tw, post, scale, s);
+            if (e != cudaErrorNotSupported)
+                return e;
+        }
     }
     if (inverse) {
         if (row) {
@@ -2277,16 +1753,6 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
             if (e != cudaErrorNotSupported)
                 return e;
         }
-        if constexpr (L == 13) {
-            const cudaError_t e = idct_col_pair_launch(d, tw, post, scale, err, 0, s);
-            if (e != cudaErrorNotSupported)
-                return e;
-        }
-        if constexpr (L == 14) {
-            const cudaError_t e = idct_col_quad_launch(d, tw, post, scale, err, 0, s);
-            if (e != cudaErrorNotSupported)
-                return e;
-        }
         return idct_launch<LineCfg<L, col_kw(L), 0>, false>(d, tw, post, d.cols / 2, scale, s);
     }
     if (row) {
@@ -2302,16 +1768,6 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
     if constexpr (L == 11) {
         const cudaError_t e =
             dct_col_tma_launch<LineCfg<L, col_kw(L), 0, 32>>(d, tw, post, scale, err, 0, s);
-        if (e != cudaErrorNotSupported)
-            return e;
-    }
-    if constexpr (L == 13 || L == 14) {
-        const cudaError_t e = dct_col_pack_launch<L - 12>(d, tw, post, scale, err, 0, s);
-        if (e != cudaErrorNotSupported)
-            return e;
-    }
-    if constexpr (L == 14) {
-        const cudaError_t e = dct_col_quad_launch(d, tw, post, scale, err, 0, s);
         if (e != cudaErrorNotSupported)
             return e;
     }

@@ -208,6 +208,8 @@ fft2d_status run_pass(const fft2d_plan_s *p, int pass, const void *in, void *out
         a.tw = p->tw_cols;
         if (p->dir == FFT2D_INVERSE && allow_scale)
             a.scale = (float)(1.0 / ((double)p->rows * (double)p->cols));
+        if (withhold)
+            a.variant = fft2d::col_selftest_variant(L, a);
         if (withhold && !fft2d::col_pass_is_tma_fed(L, a)) {
             std::snprintf(g_last_error, sizeof g_last_error,
                           "the column pass of this plan does not run on a TMA-fed kernel");
@@ -1072,7 +1074,7 @@ fft2d_status fft2d_plan_describe(fft2d_plan_t p, char *buf, int len)
         const bool tuned = i >= 0;
         if (i < 0 || i >= n)
             i = pass == FFT2D_PASS_ROWS ? fft2d::row_default_variant(L)
-                                        : fft2d::col_default_variant(L);
+                                        : fft2d::col_default_variant(L, p->cols);
         char tmp[96];
         std::snprintf(tmp, sizeof tmp, "%s(shape=%d,ept=%d,%s)", v[i].name, v[i].shape, v[i].ept,
                       tuned ? "tuned" : "default");

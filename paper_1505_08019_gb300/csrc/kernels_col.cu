@@ -355,6 +355,18 @@ cudaError_t col_launch_cluster(const PassArgs &a, cudaStream_t s)
                                                a.nst, s);
 }
 
+// Columns of 8192 and 16384 rows in two phases through an L2-resident strip
+// (col_strip.cu).
+bool col_strip_usable(const PassArgs &a) { return !a.partial; }
+
+template <int L>
+cudaError_t col_launch_strip(const PassArgs &a, cudaStream_t s)
+{
+    const StripPass p{a.in, a.out, a.ld, a.cols, a.tw, nullptr, a.scale};
+    const cudaError_t e = launch_col_strip(StripKind::C64, L, p, s);
+    return e != cudaErrorNotSupported ? e : col_launch_any<LineCfg<L, col_kw(L), 0>>(a, s);
+}
+
 bool always(const PassArgs &) { return true; }
 bool whole_stages(const PassArgs &a) { return !a.partial; }
 
@@ -447,6 +459,9 @@ struct ColVariants {
         if constexpr (L == 14)
             t.v[t.n++] = {"quadl2", PairLocal6::W, 64, col_group_usable<PairLocal6, 2>,
                           col_launch_group_l2<PairLocal6, 2>, true};
+        // two phases per 32-column strip, the intermediate in L2
+        if constexpr (L >= 13)
+            t.v[t.n++] = {"stripl2", 32, 16, col_strip_usable, col_launch_strip<L>};
         return t;
     }
     static const Variant *table(int *n)
@@ -468,7 +483,14 @@ struct ColVariants {
     // GB300 (512..4096 rows, square and 1:4 images): narrow tiles for 512 and
     // 1024 rows; the TMA pass in two groups of 6 stages with per-thread
     // stores for 2048, and with half TMA / half per-thread stores for 4096.
-    static int preferred()
+    // 8192 rows: two phases through an L2-resident strip ("stripl2") against
+    // the CTA pair ("pairl2"): 6.5 / 16.5 us for 32 columns, 40.0 / 51.4 for
+    // 1024, 157 / 164 for 4096, 312 / 314 for 8192.  16384 rows, against four
+    // CTAs ("quadl2"): 6.1 / 16.6 us for 32 columns, 81.8 / 94.4 for 1024,
+    // 323 / 329 for 4096, but 644 / 628 for 8192 and 1.28 / 1.24 ms for 16384:
+    // there the strips' four crossings of the L2 boundary cost more than the
+    // cluster's rounding to whole waves of 36 tiles.
+    static int preferred(int cols)
     {
         if constexpr (L == 9 || L == 10)
             return index_of("narrow");
@@ -477,9 +499,9 @@ struct ColVariants {
         else if constexpr (L == 12)
             return index_of("tma64");     // 61.8 vs 66.0 us for "tma32h" at 4096^2
         else if constexpr (L == 13)
-            return index_of("pairl2");    // 4-column tiles over a CTA pair (0.316 vs 0.334 ms for "pair")
+            return index_of("stripl2");
         else if constexpr (L == 14)
-            return index_of("quadl2");    // 4-column tiles over 4 CTAs (1.24 vs 1.83 ms for "quad")
+            return index_of(cols <= 4096 ? "stripl2" : "quadl2");
         else
             return 0;
     }
@@ -508,15 +530,15 @@ const Variant *col_variants(int L, int *n)
     }
 }
 
-int col_default_variant(int L)
+int col_default_variant(int L, int cols)
 {
     switch (L) {
-    case 9: return ColVariants<9>::preferred();
-    case 10: return ColVariants<10>::preferred();
-    case 11: return ColVariants<11>::preferred();
-    case 12: return ColVariants<12>::preferred();
-    case 13: return ColVariants<13>::preferred();
-    case 14: return ColVariants<14>::preferred();
+    case 9: return ColVariants<9>::preferred(cols);
+    case 10: return ColVariants<10>::preferred(cols);
+    case 11: return ColVariants<11>::preferred(cols);
+    case 12: return ColVariants<12>::preferred(cols);
+    case 13: return ColVariants<13>::preferred(cols);
+    case 14: return ColVariants<14>::preferred(cols);
     default: return 0;
     }
 }
@@ -530,7 +552,7 @@ const Variant *select_col_variant(int L, const PassArgs &a)
     const Variant *v = col_variants(L, &n);
     if (!v || n == 0)
         return nullptr;
-    int i = a.variant >= 0 && a.variant < n ? a.variant : col_default_variant(L);
+    int i = a.variant >= 0 && a.variant < n ? a.variant : col_default_variant(L, a.cols);
     if (!v[i].usable(a))
         i = 0;   // the plain kernel serves every case
     return &v[i];
@@ -542,6 +564,19 @@ cudaError_t launch_col_pass(int L, const PassArgs &a, cudaStream_t s)
 {
     const Variant *v = select_col_variant(L, a);
     return v ? v->launch(a, s) : cudaErrorInvalidValue;
+}
+
+// The strip kernel waits for nothing on the device, so the withheld-load
+// self-test of a plan that takes it runs the cluster kernel of its length.
+int col_selftest_variant(int L, const PassArgs &a)
+{
+    if (a.variant >= 0)
+        return a.variant;
+    if (L == 13)
+        return ColVariants<13>::index_of("pairl2");
+    if (L == 14)
+        return ColVariants<14>::index_of("quadl2");
+    return -1;
 }
 
 bool col_pass_is_tma_fed(int L, const PassArgs &a)

@@ -106,7 +106,7 @@ struct Variant {
 const Variant *row_variants(int L, int *n);
 const Variant *col_variants(int L, int *n);
 int row_default_variant(int L);
-int col_default_variant(int L);
+int col_default_variant(int L, int cols);
 
 // Per-size CTA shapes of the plain kernels: log2 of the rows per CTA of the
 // row pass (256 threads per CTA up to 4096-point rows) and log2 of the
@@ -267,6 +267,21 @@ cudaError_t launch_dct_pass(bool row, bool inverse, int L, const float *in, floa
                             int cols, const float2 *tw, const float2 *post, float scale, int *err,
                             cudaStream_t s, int withhold = 0);
 
+// Column pass of 2^13 or 2^14 rows in two phases through an L2-resident
+// scratch strip (col_strip.cu), complex64 or two real columns per complex
+// column (DCT-II, DCT-III).  in may equal out.  cudaErrorNotSupported
+// (nothing launched) when it does not serve these arguments.
+enum class StripKind { C64, Dct, Idct };
+struct StripPass {
+    const float2 *in;
+    float2 *out;
+    long long ld;               // row pitch in complex values
+    int cols;                   // complex columns
+    const float2 *tw, *post;    // post: DCT kinds, (cos, sin)(pi k / (2N))
+    float scale;
+};
+cudaError_t launch_col_strip(StripKind kind, int L, const StripPass &a, cudaStream_t s);
+
 // 3D tensor map over 8-byte elements: x = element within a row (xdim), y
 // (ydim rows, ystride elements apart), z (zdim blocks, zstride elements
 // apart); box box_x x box_y x box_z.  False if the driver's encoder is
@@ -291,6 +306,8 @@ int device_sm_count();
 int device_current();
 cudaError_t launch_selftest_timeout(int *err, cudaStream_t s);
 cudaError_t launch_col_pass(int L, const PassArgs &a, cudaStream_t s);
+// The variant that the withheld-load self-test runs for these arguments.
+int col_selftest_variant(int L, const PassArgs &a);
 // Whether the column-pass kernel that launch_col_pass would run for these
 // arguments is a TMA-fed one (the only kernels with the withhold self-test).
 bool col_pass_is_tma_fed(int L, const PassArgs &a);
