@@ -242,170 +242,80 @@ __global__ void __launch_bounds__(C::T, C::MINB) line_dct_kernel(const DctIO d,
 //   Z[k]   = (c + i s) ((X_a[k] + X_b[N-k]) + i (X_b[k] - X_a[N-k])),
 //   Z[N-k] = (s + i c) ((X_a[N-k] + X_b[k]) + i (X_b[N-k] - X_a[k])),
 // (c, s) = (cos, sin)(pi k / (2N)); Z[0] = z[0].
-// The un-reordering store of v[n] and v[N-1-n] (n < N/2) of complex line lb
-// (rows: real rows 2(line0+lb), +1; columns: complex column line0 + w).
-template <bool ROW>
-__device__ __forceinline__ void idct_store(const DctIO &d, long long line0, int lb, int w, int n,
-                                           float2 zn, float2 zm, float scale)
-{
-    if constexpr (ROW) {
-        const long long ra = 2 * (line0 + lb);
-        reinterpret_cast<float2 *>(d.out + ra * d.cols)[n] = make_float2(zn.x * scale, zm.x * scale);
-        reinterpret_cast<float2 *>(d.out + (ra + 1) * d.cols)[n] =
-            make_float2(zn.y * scale, zm.y * scale);
-    } else {
-        float2 *o = reinterpret_cast<float2 *>(d.out) + line0 + w;
-        o[(long long)(2 * n) * (d.cols / 2)] = make_float2(zn.x * scale, zn.y * scale);
-        o[(long long)(2 * n + 1) * (d.cols / 2)] = make_float2(zm.x * scale, zm.y * scale);
-    }
-}
+// The storage of an inverse pass on the line engine (line_fft.cuh): a load
+// brings X[k] and X[N-k] of both real lines and rotates them into Z[k]
+// (idct_pre, one side of it), a store puts v[n] where the un-reordering wants
+// it.  Every value is loaded twice, the second time from L1 or L2: that
+// replaced a pass of the whole tile through shared memory before the first
+// stages and one after the last (four barriers).
+template <int N>
+struct IdctIO {
+    static constexpr bool H16 = false, CG = false, MAPPED = true;
+    static constexpr int AXIS = -1;
+    const float *in;
+    float *out;
+    const float2 *post;
+    long long cols;
 
-// The inverse pass for any line length: the spectrum lines land in shared
-// memory in natural order, are pre-rotated in place (pairs k, N-k), run
-// through the radix-2 stages from there (conjugate rotation factors), come
-// back in natural order and leave un-reordered.
-template <class C, bool ROW>
-__global__ void __launch_bounds__(C::T, C::MINB) line_idct_kernel(const DctIO d,
+    template <bool ROW>
+    __device__ __forceinline__ float2 at(const Geo &g, int lb, int k, int w) const
+    {
+        if constexpr (ROW) {
+            const float *p = in + 2 * (g.r0 + lb) * cols + k;
+            return make_float2(ld_img(p), ld_img(p + cols));
+        } else {
+            return ld_img(reinterpret_cast<const float2 *>(in) + k * (cols / 2) + g.c0 + w);
+        }
+    }
+    template <bool ROW>
+    __device__ __forceinline__ float2 load(const Geo &g, int lb, int k, int w) const
+    {
+        const float2 z = at<ROW>(g, lb, k, w);
+        const float2 m = at<ROW>(g, lb, (N - k) & (N - 1), w);
+        const bool low = k <= N / 2;
+        const float2 cs = __ldg(post + (low ? k : N - k));
+        const float2 rot = low ? cs : make_float2(cs.y, cs.x);
+        const float ux = z.x + m.y, uy = z.y - m.x;
+        return k == 0 ? z : make_float2(rot.x * ux - rot.y * uy, rot.y * ux + rot.x * uy);
+    }
+    template <bool ROW>
+    __device__ __forceinline__ void store(const Geo &g, int lb, int n, int w, float2 v) const
+    {
+        const int x = n < N / 2 ? 2 * n : 2 * (N - 1 - n) + 1;
+        if constexpr (ROW) {
+            float *p = out + 2 * (g.r0 + lb) * cols + x;
+            p[0] = v.x;
+            p[cols] = v.y;
+        } else {
+            reinterpret_cast<float2 *>(out)[x * (cols / 2) + g.c0 + w] = v;
+        }
+    }
+};
+
+template <class C, bool ROW, bool GENERIC>
+__global__ void __launch_bounds__(C::T, C::MINB) line_idct_kernel(const IdctIO<C::N> io,
                                                                   const float2 *__restrict__ tw,
-                                                                  const float2 *__restrict__ post,
                                                                   long long nlines, float scale)
 {
-    extern __shared__ float2 sm[];
-    constexpr int HALF = C::N / 2;
-    const int tid = threadIdx.x;
-    pdl_wait();
-    const long long line0 = (long long)blockIdx.x * (ROW ? C::LB : C::W);
-    const long long nvalid = nlines - line0;
-    for (int e = tid; e < C::E; e += C::T) {
-        const int w = e & (C::W - 1);
-        const int k = (e >> C::KW) & (C::N - 1);
-        const int lb = e >> (C::L + C::KW);
-        float2 z = make_float2(0.f, 0.f);
-        if (ROW ? lb < nvalid : w < nvalid) {
-            if constexpr (ROW) {
-                const long long ra = 2 * (line0 + lb);
-                z = make_float2(ld_img(d.in + ra * d.cols + k), ld_img(d.in + (ra + 1) * d.cols + k));
-            } else {
-                z = ld_img(reinterpret_cast<const float2 *>(d.in) + (long long)k * (d.cols / 2) +
-                          line0 + w);
-            }
-        }
-        sm[e] = z;
-    }
-    __syncthreads();
-    // pre-rotation: item q -> line block / column and k in [0, N/2); k = 0
-    // also handles k = N/2
-#pragma unroll
-    for (int t = 0; t < C::EPT / 2; t++) {
-        const int q = tid + t * C::T;
-        const int w = ROW ? 0 : q & (C::W - 1);
-        const int rest = ROW ? q : q >> C::KW;
-        const int lb = ROW ? rest / HALF : 0;
-        const int k = rest % HALF;
-        float2 *line = sm + ((long long)lb << (C::L + C::KW)) + w;
-        float2 yk, yp;
-        if (k == 0) {
-            const float2 zh = line[HALF << C::KW];
-            idct_pre(zh, zh, __ldg(post + HALF), yk, yp);
-            line[HALF << C::KW] = yk;
-        } else {
-            idct_pre(line[k << C::KW], line[(C::N - k) << C::KW], __ldg(post + k), yk, yp);
-            line[k << C::KW] = yk;
-            line[(C::N - k) << C::KW] = yp;
-        }
-    }
-    __syncthreads();
-    float2 a[C::EPT];
-    if constexpr (C::NG == 1) {
-        using G0 = Grp<C, 0>;
-#pragma unroll
-        for (int v = 0; v < G0::V; v++) {
-            const int u = tid + v * C::T;
-            const int w = u & (C::W - 1);
-            const int lb = u >> C::KW;
-#pragma unroll
-            for (int r = 0; r < G0::R; r++)
-                a[v * G0::R + r] = sm[(((lb << C::L) | brev_c(r, G0::G)) << C::KW) | w];
-            run_stages<C, 0, false>(a, v, 0, tw, C::L);
-            if (ROW ? lb >= nvalid : w >= nvalid)
-                continue;
-#pragma unroll
-            for (int n = 0; n < HALF; n++)
-                idct_store<ROW>(d, line0, lb, w, n, a[v * G0::R + n], a[v * G0::R + C::N - 1 - n],
-                                scale);
-        }
-    } else {
-        group_first_smem<C, false>(a, sm, tw, C::L);
-        __syncthreads();
-        if constexpr (C::NG >= 3) {
-            group_smem<C, 1, false>(a, sm, tw, C::L);
-            __syncthreads();
-        }
-        if constexpr (C::NG >= 4) {
-            group_smem<C, 2, false>(a, sm, tw, C::L);
-            __syncthreads();
-        }
-        using Gl = Grp<C, C::NG - 1>;
-#pragma unroll
-        for (int v = 0; v < Gl::V; v++) {
-            const int u = tid + v * C::T;
-            const int w = u & (C::W - 1);
-            const int u2 = u >> C::KW;
-            const int lo = u2 & ((1 << Gl::S0) - 1);
-            const int lb = u2 >> Gl::S0;
-#pragma unroll
-            for (int r = 0; r < Gl::R; r++)
-                a[v * Gl::R + r] = sm[sidx<C>(lb, lo | (r << Gl::S0), w)];
-        }
-#pragma unroll
-        for (int v = 0; v < Gl::V; v++) {
-            const int u = tid + v * C::T;
-            const int lo = (u >> C::KW) & ((1 << Gl::S0) - 1);
-            run_stages<C, C::NG - 1, false>(a, v, lo, tw, C::L);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int v = 0; v < Gl::V; v++) {
-            const int u = tid + v * C::T;
-            const int w = u & (C::W - 1);
-            const int u2 = u >> C::KW;
-            const int lo = u2 & ((1 << Gl::S0) - 1);
-            const int lb = u2 >> Gl::S0;
-#pragma unroll
-            for (int r = 0; r < Gl::R; r++)
-                sm[((((lb << C::L) | lo | (r << Gl::S0))) << C::KW) | w] = a[v * Gl::R + r];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int t = 0; t < C::EPT / 2; t++) {
-            const int q = tid + t * C::T;
-            const int w = ROW ? 0 : q & (C::W - 1);
-            const int rest = ROW ? q : q >> C::KW;
-            const int lb = ROW ? rest / HALF : 0;
-            const int n = rest % HALF;
-            if (ROW ? lb >= nvalid : w >= nvalid)
-                continue;
-            const float2 *line = sm + ((long long)lb << (C::L + C::KW)) + w;
-            idct_store<ROW>(d, line0, lb, w, n, line[n << C::KW], line[(C::N - 1 - n) << C::KW],
-                            scale);
-        }
-    }
+    const long long l0 = (long long)blockIdx.x * (ROW ? C::LB : C::W);
+    line_fft<C, ROW, GENERIC>(io, ROW ? Geo{l0, 1, 0, 0} : Geo{0, 1, l0, 0}, tw, scale, C::L,
+                              nlines - l0);
 }
 
 template <class C, bool ROW>
 cudaError_t idct_launch(const DctIO &d, const float2 *tw, const float2 *post, long long nlines,
                         float scale, cudaStream_t s)
 {
-    auto k = line_idct_kernel<C, ROW>;
-    constexpr int bytes = C::E * 8;
+    const long long per = ROW ? C::LB : C::W;
+    auto k = nlines % per ? line_idct_kernel<C, ROW, true> : line_idct_kernel<C, ROW, false>;
+    constexpr int bytes = C::SMEM_BYTES;
     if (bytes > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess)
             return e;
     }
-    const long long per = ROW ? C::LB : C::W;
-    const unsigned grid = (unsigned)((nlines + per - 1) / per);
-    return launch_chained(k, (unsigned)grid, C::T, bytes, s, 1, d, tw, post, nlines, scale);
+    return launch_chained(k, dim3((unsigned)((nlines + per - 1) / per)), C::T, bytes, s, 1,
+                          IdctIO<C::N>{d.in, d.out, post, d.cols}, tw, nlines, scale);
 }
 
 // The last stage group of a line: unit lo (0 <= lo < M = 2^S0) holds rows
@@ -1693,6 +1603,27 @@ cudaError_t dct_col_strip(bool inverse, int L, const DctIO &d, const float2 *tw,
     return launch_col_strip(inverse ? StripKind::Idct : StripKind::Dct, L, p, s);
 }
 
+// Tile of the generic column kernels: log2 of the complex values per CTA, 0
+// for the TMA-fed kernel of the length.  As in the complex64 pass (see
+// kernels_col.cu), small CTAs win while about one per SM covers the image.
+// Measured with 2^12 (128 CTAs at most) against the earlier choice, forward /
+// inverse: 128 rows 3.0 / 2.7 against 4.5 / 7.3 us, 256 rows 3.2 / 3.2
+// against 4.7 / 7.4, 512 rows 3.9 / 3.6 against 5.4 / 8.2, 1024 rows 4.4 / 4.5
+// against 9.1 / 12.3, 2048 rows (TMA-fed before) 5.9 / 6.8 against 11.5 / 11.2,
+// 4096 rows 8.8 against 11.6 (inverse 11.4 / 11.5: stays).  2^13 in the next
+// range: 1024 x 8192 20.7 / 20.8 against 23.4 / 38.5, 2048 x 1024 7.3 / 7.3
+// against 11.8 / 11.5, 4096 x 512 10.0 against 11.8.
+template <int L>
+int dct_col_tile(bool inverse, long long cols)
+{
+    if constexpr (L < 6 || L > 12)
+        return 13;
+    if (L <= 8 || (L == 9 && !inverse))
+        return 12;
+    const int small = L == 12 && inverse ? 0 : col_small_tile((cols / 2) << L);
+    return small ? small : L <= 10 ? 13 : 0;
+}
+
 template <int L>
 cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *tw,
                          const float2 *post, float scale, int *err, int withhold, cudaStream_t s)
@@ -1743,15 +1674,24 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
             return idct_launch<LineCfg<L, 0, row_kb(L)>, true>(d, tw, post, d.rows / 2, scale, s);
         }
         if constexpr (L == 12) {
-            const cudaError_t e = idct_col_tma64_launch(d, tw, post, scale, err, 0, s);
-            if (e != cudaErrorNotSupported)
-                return e;
+            if (!dct_col_tile<L>(true, d.cols)) {
+                const cudaError_t e = idct_col_tma64_launch(d, tw, post, scale, err, 0, s);
+                if (e != cudaErrorNotSupported)
+                    return e;
+            }
         }
         if constexpr (L == 11) {
-            const cudaError_t e =
-                idct_col_tma_launch<LineCfg<L, col_kw(L), 0, 32>>(d, tw, post, scale, err, 0, s);
-            if (e != cudaErrorNotSupported)
-                return e;
+            if (!dct_col_tile<L>(true, d.cols)) {
+                const cudaError_t e =
+                    idct_col_tma_launch<LineCfg<L, col_kw(L), 0, 32>>(d, tw, post, scale, err, 0, s);
+                if (e != cudaErrorNotSupported)
+                    return e;
+            }
+        }
+        if constexpr (L >= 6 && L <= 12) {
+            if (dct_col_tile<L>(true, d.cols) == 12)
+                return idct_launch<LineCfg<L, 12 - L, 0>, false>(d, tw, post, d.cols / 2, scale, s);
+            return idct_launch<LineCfg<L, 13 - L, 0>, false>(d, tw, post, d.cols / 2, scale, s);
         }
         return idct_launch<LineCfg<L, col_kw(L), 0>, false>(d, tw, post, d.cols / 2, scale, s);
     }
@@ -1761,15 +1701,24 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
         return dct_launch<LineCfg<L, 0, row_kb(L)>, true>(d, tw, post, d.rows / 2, scale, s);
     }
     if constexpr (L == 12) {
-        const cudaError_t e = dct_col_tma64_launch(d, tw, post, scale, err, 0, s);
-        if (e != cudaErrorNotSupported)
-            return e;
+        if (!dct_col_tile<L>(false, d.cols)) {
+            const cudaError_t e = dct_col_tma64_launch(d, tw, post, scale, err, 0, s);
+            if (e != cudaErrorNotSupported)
+                return e;
+        }
     }
     if constexpr (L == 11) {
-        const cudaError_t e =
-            dct_col_tma_launch<LineCfg<L, col_kw(L), 0, 32>>(d, tw, post, scale, err, 0, s);
-        if (e != cudaErrorNotSupported)
-            return e;
+        if (!dct_col_tile<L>(false, d.cols)) {
+            const cudaError_t e =
+                dct_col_tma_launch<LineCfg<L, col_kw(L), 0, 32>>(d, tw, post, scale, err, 0, s);
+            if (e != cudaErrorNotSupported)
+                return e;
+        }
+    }
+    if constexpr (L >= 6 && L <= 12) {
+        if (dct_col_tile<L>(false, d.cols) == 12)
+            return dct_launch<LineCfg<L, 12 - L, 0>, false>(d, tw, post, d.cols / 2, scale, s);
+        return dct_launch<LineCfg<L, 13 - L, 0>, false>(d, tw, post, d.cols / 2, scale, s);
     }
     return dct_launch<LineCfg<L, col_kw(L), 0>, false>(d, tw, post, d.cols / 2, scale, s);
 }

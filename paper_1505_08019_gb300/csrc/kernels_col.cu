@@ -385,6 +385,7 @@ struct ColVariants {
     static constexpr bool HASNARROW = L >= 5 && KWN >= 2;
 
     using Narrow = LineCfg<L, (KWN >= 0 ? KWN : 0), 0>;
+    using Fine = LineCfg<L, (L <= 12 ? 12 - L : 0), 0>;
     // cluster shapes: W = 8 over 2 (2048 rows) or 4 (4096 rows) CTAs;
     // W = 4 over 2 or 4 CTAs for 8192 and 16384 rows
     static constexpr int CKW = L <= 12 ? 3 : 2;
@@ -459,6 +460,9 @@ struct ColVariants {
         if constexpr (L == 14)
             t.v[t.n++] = {"quadl2", PairLocal6::W, 64, col_group_usable<PairLocal6, 2>,
                           col_launch_group_l2<PairLocal6, 2>, true};
+        // 4096 values (256 threads) per CTA, for images of few columns
+        if constexpr (L == 10 || L == 11)
+            t.v[t.n++] = {"fine", Fine::W, 16, whole_stages, col_launch_any<Fine>};
         // two phases per 32-column strip, the intermediate in L2
         if constexpr (L >= 13)
             t.v[t.n++] = {"stripl2", 32, 16, col_strip_usable, col_launch_strip<L>};
@@ -479,10 +483,18 @@ struct ColVariants {
                 return i;
         return 0;
     }
-    // The default per column length, from timings of every variant on a
-    // GB300 (512..4096 rows, square and 1:4 images): narrow tiles for 512 and
-    // 1024 rows; the TMA pass in two groups of 6 stages with per-thread
-    // stores for 2048, and with half TMA / half per-thread stores for 4096.
+    // The default per column length and width, from timings of every variant
+    // on a GB300 (images in turn, 16 to 8192 columns).  Small CTAs win as long
+    // as they fit the 152 SMs about once: the pass is then one CTA's latency.
+    // 128 and 256 rows: "narrow" (4096 values) at every width, 2.6 / 3.2 us
+    // and 3.0 / 4.2 for "plain" up to 2048 columns.  512 rows: "narrow".  1024
+    // rows: "fine" for up to 128 of its CTAs (512 columns), 3.8 against 4.9 us
+    // for "narrow", which wins from 1024 columns (5.2 / 5.5).  2048 rows:
+    // "fine" up to 128 CTAs (256 columns), 5.3 us, "narrow" up to 128 (512
+    // columns), 6.0, against 8.1 - 8.5 for the TMA pass in two groups of 6
+    // stages with per-thread stores ("tma64st"), which wins from 1024 columns
+    // (9.6 / 10.8; 16.9 / 21.1 at 2048).  4096 rows: the TMA pass with half
+    // TMA / half per-thread stores ("tma64").
     // 8192 rows: two phases through an L2-resident strip ("stripl2") against
     // the CTA pair ("pairl2"): 6.5 / 16.5 us for 32 columns, 40.0 / 51.4 for
     // 1024, 157 / 164 for 4096, 312 / 314 for 8192.  16384 rows, against four
@@ -492,10 +504,14 @@ struct ColVariants {
     // cluster's rounding to whole waves of 36 tiles.
     static int preferred(int cols)
     {
-        if constexpr (L == 9 || L == 10)
+        if constexpr (L >= 7 && L <= 9)
             return index_of("narrow");
+        else if constexpr (L == 10)
+            return index_of(cols <= 128 * Fine::W ? "fine" : "narrow");
         else if constexpr (L == 11)
-            return index_of("tma64st");   // 20.7 vs 22.5 us for "tma32st" at 2048^2
+            return index_of(cols <= 128 * Fine::W     ? "fine"
+                            : cols <= 128 * Narrow::W ? "narrow"
+                                                      : "tma64st");
         else if constexpr (L == 12)
             return index_of("tma64");     // 61.8 vs 66.0 us for "tma32h" at 4096^2
         else if constexpr (L == 13)
@@ -533,6 +549,8 @@ const Variant *col_variants(int L, int *n)
 int col_default_variant(int L, int cols)
 {
     switch (L) {
+    case 7: return ColVariants<7>::preferred(cols);
+    case 8: return ColVariants<8>::preferred(cols);
     case 9: return ColVariants<9>::preferred(cols);
     case 10: return ColVariants<10>::preferred(cols);
     case 11: return ColVariants<11>::preferred(cols);
@@ -566,12 +584,15 @@ cudaError_t launch_col_pass(int L, const PassArgs &a, cudaStream_t s)
     return v ? v->launch(a, s) : cudaErrorInvalidValue;
 }
 
-// The strip kernel waits for nothing on the device, so the withheld-load
-// self-test of a plan that takes it runs the cluster kernel of its length.
+// The strip kernel and the small-tile kernels wait for nothing on the device,
+// so the withheld-load self-test of a plan that takes them by default runs the
+// TMA-fed kernel of its column length.
 int col_selftest_variant(int L, const PassArgs &a)
 {
     if (a.variant >= 0)
         return a.variant;
+    if (L == 11)
+        return ColVariants<11>::index_of("tma64st");
     if (L == 13)
         return ColVariants<13>::index_of("pairl2");
     if (L == 14)

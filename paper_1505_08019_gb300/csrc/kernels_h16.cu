@@ -170,6 +170,12 @@ cudaError_t h16_launch_col_group(const H16PassArgs &a, cudaStream_t s)
     return e != cudaSuccess ? e : f;
 }
 
+template <class C>
+cudaError_t h16_launch_col_tile(const H16PassArgs &a, cudaStream_t s)
+{
+    return a.cols % C::W ? h16_launch<C, false, true>(a, s) : h16_launch<C, false, false>(a, s);
+}
+
 template <int L>
 cudaError_t h16_dispatch(bool row, const H16PassArgs &a, cudaStream_t s)
 {
@@ -186,6 +192,18 @@ cudaError_t h16_dispatch(bool row, const H16PassArgs &a, cudaStream_t s)
         }
     }
     using C = LineCfg<L, col_kw(L), 0>;
+    if constexpr (L >= 7 && L <= 12) {
+        // few columns: small tiles (col_small_tile).  Whole transform, before
+        // and here: 128x2048 6.6 / 5.6 us, 256x2048 7.9 / 7.3, 512x1024 8.3 /
+        // 7.8, 1024x512 11.7 / 8.3, 1024x1024 12.6 / 10.2 (2^13), 2048x256 12.6
+        // / 8.9, 2048x512 15.0 / 11.9 (2^13), 4096x128 18.4 / 13.6, 4096x256
+        // 18.8 / 14.9 (2^13)
+        const int tile = L == 7 ? 12 : col_small_tile((long long)a.cols << L);
+        if (tile == 12)
+            return h16_launch_col_tile<LineCfg<L, 12 - L, 0>>(a, s);
+        if (tile == 13)
+            return h16_launch_col_tile<LineCfg<L, 13 - L, 0>>(a, s);
+    }
     if constexpr (L == 12) {
         const cudaError_t e = h16_launch_col_tma<L>(a, s);
         if (e != cudaErrorNotSupported)
@@ -206,7 +224,7 @@ cudaError_t h16_dispatch(bool row, const H16PassArgs &a, cudaStream_t s)
             return launch_cluster_kernel<CC, StoreH16>(io, a.tw, a.cols, a.ld, a.scale, a.nst, s);
         }
     }
-    return a.cols % C::W ? h16_launch<C, false, true>(a, s) : h16_launch<C, false, false>(a, s);
+    return h16_launch_col_tile<C>(a, s);
 }
 
 // complex64 -> half2 + one exponent per row (the pass exponent rule: the

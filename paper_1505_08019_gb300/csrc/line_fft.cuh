@@ -225,6 +225,7 @@ __device__ __forceinline__ void run_stages(float2 (&a)[C::EPT], int v, int lo,
 struct StoreC64 {
     static constexpr bool H16 = false;
     static constexpr bool CG = false;   // load through L2 only (see small.cu)
+    static constexpr bool MAPPED = false;   // load and store through the members load / store
     static constexpr int AXIS = -1;
     using T = float2;
     const float2 *in;
@@ -237,6 +238,7 @@ template <int IA = -1>
 struct StoreH16T {
     static constexpr bool H16 = true;
     static constexpr bool CG = false;
+    static constexpr bool MAPPED = false;
     static constexpr int AXIS = IA;
     using T = __half2;
     const __half2 *in;
@@ -303,8 +305,10 @@ template <class IO, bool ROW>
 __device__ __forceinline__ float2 load_pix(const IO &io, const Geo &g, int lb, int i, int w,
                                            float f = 0.f)
 {
-    const long long k = pix<ROW>(g, lb, i, w);
-    if constexpr (IO::H16) {
+    if constexpr (IO::MAPPED) {
+        return io.template load<ROW>(g, lb, i, w);
+    } else if constexpr (IO::H16) {
+        const long long k = pix<ROW>(g, lb, i, w);
         __half2 h;
         if constexpr (IO::CG)
             h = __ldcg(io.in + k);
@@ -315,9 +319,9 @@ __device__ __forceinline__ float2 load_pix(const IO &io, const Geo &g, int lb, i
             f = in_factor<IO, ROW>(io, g, lb, i, w);
         return make_float2(q.x * f, q.y * f);
     } else if constexpr (IO::CG) {
-        return __ldcg(io.in + k);
+        return __ldcg(io.in + pix<ROW>(g, lb, i, w));
     } else {
-        return ld_stream(io.in + k);
+        return ld_stream(io.in + pix<ROW>(g, lb, i, w));
     }
 }
 
@@ -388,13 +392,15 @@ __device__ __forceinline__ void store_units(float2 (&a)[C::EPT], const IO &io, c
         for (int r = 0; r < Gp::R; r++) {
             const int p = pos(v, r) & (C::N - 1);
             const float2 x = a[v * Gp::R + r];
-            const long long k = pix<ROW>(g, lb, p, w);
-            if constexpr (IO::H16) {
+            if constexpr (IO::MAPPED) {
+                io.template store<ROW>(g, lb, p, w, make_float2(x.x * f, x.y * f));
+            } else if constexpr (IO::H16) {
+                const long long k = pix<ROW>(g, lb, p, w);
                 io.out[k] = __floats2half2_rn(x.x * f, x.y * f);
                 if (p == 0)
                     io.out_exp[ROW ? g.r0 + lb : g.c0 + w] = e;
             } else {
-                io.out[k] = make_float2(x.x * f, x.y * f);
+                io.out[pix<ROW>(g, lb, p, w)] = make_float2(x.x * f, x.y * f);
             }
         }
     }

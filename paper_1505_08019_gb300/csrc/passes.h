@@ -118,6 +118,16 @@ constexpr int col_kw(int L)
     return L >= 10 ? 14 - L : (13 - L < 4 ? 4 : (13 - L > 6 ? 6 : 13 - L));
 }
 
+// Column passes over few values: log2 of the values per CTA tile (256 or 512
+// threads x 16) that covers them with at most 128 CTAs, 0 when there are more.
+// Below that line a pass is the latency of one CTA on fewer SMs than there
+// are, and the smaller CTA is the faster one; above it the wider row segments
+// of the larger tiles win (timings beside each dispatch).
+constexpr int col_small_tile(long long values)
+{
+    return values <= 128ll << 12 ? 12 : values <= 128ll << 13 ? 13 : 0;
+}
+
 // Values per thread of the TMA column kernel: 32 for tiles of 2^14 values
 // (512 threads of up to 128 registers), 16 below.
 constexpr int col_tma_ept(int L) { return L >= 10 ? 32 : 16; }
