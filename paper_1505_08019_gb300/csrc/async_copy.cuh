@@ -32,13 +32,6 @@ __device__ __forceinline__ void pdl_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Let the next chained kernel in as soon as every CTA of this one has called
-// this or left: its CTAs take SMs over as they drain and wait in pdl_wait().
-__device__ __forceinline__ void pdl_trigger()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // Image loads that stay behind pdl_wait() (the read-only path need not).
 __device__ __forceinline__ float ld_img(const float *p)
 {

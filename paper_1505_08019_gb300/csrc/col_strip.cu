@@ -24,8 +24,7 @@
 // whose items alternate in the grid (reads of the image from HBM beside
 // writes to it); a chunk is kChunk strips, so that the two chunks of scratch
 // in use stay in L2.  The kernel boundary is the only synchronisation:
-// chained launches (launch_chained, with an early trigger, so the next
-// launch's CTAs take the SMs over as they drain).  One persistent launch whose
+// chained launches (launch_chained).  One persistent launch whose
 // items waited for counters published with release increments took 0.84 -
 // 0.94 ms where this takes 0.69 (16384^2 inverse DCT): every publication waits
 // until the item's scattered stores are performed.
@@ -125,7 +124,7 @@ __global__ void __launch_bounds__(256, 4) col_strip_kernel(const StripArgs g)
     __shared__ float2 tw1[S::NA];            // stages 1 .. LA
     __shared__ float2 tw2[2 * NB];           // stages LA+1 .. L of the item's two lo
     const int tid = threadIdx.x;
-    pdl_trigger();
+
     pdl_wait();
     // items of the two phases alternate as long as there are both
     const int both = 2 * (g.items[0] < g.items[1] ? g.items[0] : g.items[1]);

@@ -37,6 +37,7 @@
 //  * col_strip.cu: columns of 2^13 and 2^14 points, in two phases through a
 //    scratch strip in L2.
 #include <cmath>
+#include <type_traits>
 
 #include "dct_math.cuh"
 #include "line_fft.cuh"
@@ -1608,17 +1609,21 @@ cudaError_t dct_col_strip(bool inverse, int L, const DctIO &d, const float2 *tw,
 // kernels_col.cu), small CTAs win while about one per SM covers the image.
 // Measured with 2^12 (128 CTAs at most) against the earlier choice, forward /
 // inverse: 128 rows 3.0 / 2.7 against 4.5 / 7.3 us, 256 rows 3.2 / 3.2
-// against 4.7 / 7.4, 512 rows 3.9 / 3.6 against 5.4 / 8.2, 1024 rows 4.4 / 4.5
+// against 4.7 / 7.4, 512 rows 3.5 / 3.4 (two
+// groups, 5 + 4 stages, 32 values a thread) against 5.4 / 8.2, 1024 rows 4.4 / 4.5
 // against 9.1 / 12.3, 2048 rows (TMA-fed before) 5.9 / 6.8 against 11.5 / 11.2,
 // 4096 rows 8.8 against 11.6 (inverse 11.4 / 11.5: stays).  2^13 in the next
 // range: 1024 x 8192 20.7 / 20.8 against 23.4 / 38.5, 2048 x 1024 7.3 / 7.3
 // against 11.8 / 11.5, 4096 x 512 10.0 against 11.8.
 template <int L>
+using DctTile12 = typename std::conditional<L == 9, LineCfg<9, 3, 0, 32, 5>,
+                                            LineCfg<L, (L <= 12 ? 12 - L : 0), 0>>::type;
+template <int L>
 int dct_col_tile(bool inverse, long long cols)
 {
     if constexpr (L < 6 || L > 12)
         return 13;
-    if (L <= 8 || (L == 9 && !inverse))
+    if (L <= 9)
         return 12;
     const int small = L == 12 && inverse ? 0 : col_small_tile((cols / 2) << L);
     return small ? small : L <= 10 ? 13 : 0;
@@ -1690,7 +1695,7 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
         }
         if constexpr (L >= 6 && L <= 12) {
             if (dct_col_tile<L>(true, d.cols) == 12)
-                return idct_launch<LineCfg<L, 12 - L, 0>, false>(d, tw, post, d.cols / 2, scale, s);
+                return idct_launch<DctTile12<L>, false>(d, tw, post, d.cols / 2, scale, s);
             return idct_launch<LineCfg<L, 13 - L, 0>, false>(d, tw, post, d.cols / 2, scale, s);
         }
         return idct_launch<LineCfg<L, col_kw(L), 0>, false>(d, tw, post, d.cols / 2, scale, s);
@@ -1717,7 +1722,7 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
     }
     if constexpr (L >= 6 && L <= 12) {
         if (dct_col_tile<L>(false, d.cols) == 12)
-            return dct_launch<LineCfg<L, 12 - L, 0>, false>(d, tw, post, d.cols / 2, scale, s);
+            return dct_launch<DctTile12<L>, false>(d, tw, post, d.cols / 2, scale, s);
         return dct_launch<LineCfg<L, 13 - L, 0>, false>(d, tw, post, d.cols / 2, scale, s);
     }
     return dct_launch<LineCfg<L, col_kw(L), 0>, false>(d, tw, post, d.cols / 2, scale, s);

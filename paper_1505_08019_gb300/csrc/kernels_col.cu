@@ -386,6 +386,7 @@ struct ColVariants {
 
     using Narrow = LineCfg<L, (KWN >= 0 ? KWN : 0), 0>;
     using Fine = LineCfg<L, (L <= 12 ? 12 - L : 0), 0>;
+    using Fine5 = LineCfg<9, 3, 0, 32, 5>;
     // cluster shapes: W = 8 over 2 (2048 rows) or 4 (4096 rows) CTAs;
     // W = 4 over 2 or 4 CTAs for 8192 and 16384 rows
     static constexpr int CKW = L <= 12 ? 3 : 2;
@@ -463,6 +464,9 @@ struct ColVariants {
         // 4096 values (256 threads) per CTA, for images of few columns
         if constexpr (L == 10 || L == 11)
             t.v[t.n++] = {"fine", Fine::W, 16, whole_stages, col_launch_any<Fine>};
+        // 512 rows in two groups (5 + 4), 128 threads x 32 values
+        if constexpr (L == 9)
+            t.v[t.n++] = {"fine32g5", Fine5::W, 32, whole_stages, col_launch_any<Fine5>};
         // two phases per 32-column strip, the intermediate in L2
         if constexpr (L >= 13)
             t.v[t.n++] = {"stripl2", 32, 16, col_strip_usable, col_launch_strip<L>};
@@ -487,7 +491,9 @@ struct ColVariants {
     // on a GB300 (images in turn, 16 to 8192 columns).  Small CTAs win as long
     // as they fit the 152 SMs about once: the pass is then one CTA's latency.
     // 128 and 256 rows: "narrow" (4096 values) at every width, 2.6 / 3.2 us
-    // and 3.0 / 4.2 for "plain" up to 2048 columns.  512 rows: "narrow".  1024
+    // and 3.0 / 4.2 for "plain" up to 2048 columns.  512 rows: "fine32g5"
+    // at every width, 2.9 / 3.5 us for "narrow" up to 1024 columns, 13.6 / 15.7
+    // at 8192: one exchange instead of two.  1024
     // rows: "fine" for up to 128 of its CTAs (512 columns), 3.8 against 4.9 us
     // for "narrow", which wins from 1024 columns (5.2 / 5.5).  2048 rows:
     // "fine" up to 128 CTAs (256 columns), 5.3 us, "narrow" up to 128 (512
@@ -504,8 +510,10 @@ struct ColVariants {
     // cluster's rounding to whole waves of 36 tiles.
     static int preferred(int cols)
     {
-        if constexpr (L >= 7 && L <= 9)
+        if constexpr (L == 7 || L == 8)
             return index_of("narrow");
+        else if constexpr (L == 9)
+            return index_of("fine32g5");
         else if constexpr (L == 10)
             return index_of(cols <= 128 * Fine::W ? "fine" : "narrow");
         else if constexpr (L == 11)
