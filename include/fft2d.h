@@ -302,9 +302,11 @@ FFT2D_API fft2d_status fft2d_exec_host_many_async(int n, const fft2d_plan_t *pla
  * overlap).  Images are grouped by axis length and direction: one launch per
  * group runs the row pass of all its images (a job table travels as a kernel
  * parameter), then one launch per group the column pass -- a handful of
- * launches for any number of images.  Lines of 8192 and 16384 points run
- * each image's single-image pass instead, on
- * the group's internal stream.  Every image's result is bit for bit the one
+ * launches for any number of images.  In a batch of up to 2^23 pixels one
+ * launch per pass serves all lengths (columns of more than 512 rows only
+ * while they are few) whose variant was neither tuned nor forced.  Lines of
+ * 8192 and 16384 points run each image's single-image pass instead, on the
+ * group's internal stream.  Every image's result is bit for bit the one
  * fft2d_exec gives.  complex64 plans only.
  */
 FFT2D_API fft2d_status fft2d_exec_batched(int n, const fft2d_plan_t *plans, const void *const *in,

@@ -517,159 +517,248 @@ cudaError_t stream_wait_lanes(BatchLanes &bl, cudaStream_t to)
     return e;
 }
 
-// Run the grouped passes of a batch.  With `timing` set, every (pass, L,
-// direction) group is launched once per variant and timed on `st`, and the
-// fastest variant per (pass, L) is recorded (the batch autotuner);
-// otherwise each group runs once with its chosen variant, the groups of a
-// pass spread over the device's internal lanes.
-fft2d_status batched_impl(int n, const fft2d_plan_t *plans, const void *const *in,
-                          void *const *out, cudaStream_t st, bool timing)
+// One image's job of a pass (rows: in -> out; columns: in place on out).
+fft2d::BatchJob batch_job(const fft2d_plan_s *p, bool row, const void *in, void *out)
 {
-    fft2d::NvtxRange range(timing ? "fft2d batched autotune" : "fft2d batched");
-    BatchLanes *bl = nullptr;
-    std::unique_lock<std::mutex> lanes_lock;
-    if (!timing && n > 0) {
-        bl = batch_lanes(plans[0]->device, st);
-        if (!bl)
-            return FFT2D_ERR_OOM;
-        lanes_lock = std::unique_lock<std::mutex>(bl->mu);
-        cudaError_t e = batch_lanes_prepare(*bl);
-        if (e == cudaSuccess)
-            e = lanes_wait_stream(*bl, st);
-        if (e != cudaSuccess)
-            return cuda_fail(e, "batch lanes");
-    }
-    int group = 0;
+    fft2d::BatchJob j;
+    j.in = static_cast<const float2 *>(row ? in : out);
+    j.out = static_cast<float2 *>(out);
+    j.tw = row ? p->tw_rows : p->tw_cols;
+    j.ld = p->cols;
+    j.lines = row ? p->rows : p->cols;
+    j.first_cta = 0;
+    j.scale = (!row && p->dir == FFT2D_INVERSE)
+                  ? (float)(1.0 / ((double)p->rows * (double)p->cols))
+                  : 1.0f;
+    j.L = row ? p->Lc : p->Lr;
+    return j;
+}
+
+// Call launch(table, L, first image) for every (L, direction) group of a pass
+// whose length `want` accepts, at most kBatchTmaMaxJobs images at a time.
+template <class Want, class Launch>
+fft2d_status batch_groups(int n, const fft2d_plan_t *plans, const void *const *in,
+                          void *const *out, bool row, Want want, Launch launch)
+{
     static thread_local fft2d::BatchTable table;
+    for (int L = 1; L <= 14; L++) {
+        if (!want(L))
+            continue;
+        for (int dir = -1; dir <= 1; dir += 2) {
+            table.n = 0;
+            int first = -1;
+            for (int i = 0; i <= n; i++) {
+                if ((i == n || table.n == fft2d::kBatchTmaMaxJobs) && table.n > 0) {
+                    const fft2d_status s = launch(table, L, first);
+                    if (s != FFT2D_OK)
+                        return s;
+                    table.n = 0;
+                }
+                if (i == n)
+                    break;
+                const fft2d_plan_s *p = plans[i];
+                if (p->Lr == 0 || p->Lc == 0 || (row ? p->Lc : p->Lr) != L || p->dir != dir)
+                    continue;
+                if (first < 0)
+                    first = i;
+                table.job[table.n++] = batch_job(p, row, in[i], out[i]);
+            }
+        }
+    }
+    return FFT2D_OK;
+}
+
+// Run the grouped passes of a batch.  A pass's lengths split in two: those of
+// the launch for any length (fft2d::batch_any, unless a variant was tuned or
+// forced for the length), and the rest, one launch per (length, direction)
+// spread over the device's internal lanes.  A pass without a rest needs no
+// lanes and runs on the caller's stream.
+fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in,
+                         void *const *out, cudaStream_t st)
+{
+    fft2d::NvtxRange range("fft2d batched");
+    if (n == 0)
+        return FFT2D_OK;
+    const int device = plans[0]->device;
+    long long values[2][15] = {}, total = 0;
+    for (int i = 0; i < n; i++) {
+        const fft2d_plan_s *p = plans[i];
+        if (p->Lr == 0 || p->Lc == 0)
+            continue;
+        total += (long long)p->rows * p->cols;
+        values[0][p->Lc] += (long long)p->rows * p->cols;
+        values[1][p->Lr] += (long long)p->rows * p->cols;
+    }
+    bool any[2][15] = {}, some_any[2] = {}, some_rest[2] = {};
+    {
+        std::lock_guard<std::mutex> lock(g_tune_mu);
+        load_tune_file_locked(device);
+        for (int pass = 0; pass < 2; pass++)
+            for (int L = 1; L <= 14; L++) {
+                if (values[pass][L] == 0)
+                    continue;
+                any[pass][L] = fft2d::batch_any(pass == FFT2D_PASS_ROWS, L, values[pass][L], total) &&
+                               !g_tuned.count(std::make_tuple(device, pass + 2, L, 0));
+                (any[pass][L] ? some_any : some_rest)[pass] = true;
+            }
+    }
+    // every job of the pass's launch for any length, on stream s
+    auto run_any = [&](int pass, cudaStream_t s) {
+        static thread_local fft2d::BatchTable table;
+        const bool row = pass == FFT2D_PASS_ROWS;
+        table.n = 0;
+        for (int i = 0; i <= n; i++) {
+            if ((i == n || table.n == fft2d::kBatchMaxJobs) && table.n > 0) {
+                const cudaError_t e = fft2d::launch_batch_any(row, table, s);
+                if (e != cudaSuccess)
+                    return cuda_fail(e, "batched pass");
+                table.n = 0;
+            }
+            if (i == n)
+                break;
+            const fft2d_plan_s *p = plans[i];
+            if (p->Lr > 0 && p->Lc > 0 && any[pass][row ? p->Lc : p->Lr])
+                table.job[table.n++] = batch_job(p, row, in[i], out[i]);
+        }
+        return FFT2D_OK;
+    };
+    fft2d_status result = FFT2D_OK;
+    if (!some_rest[0] && some_any[0])
+        result = run_any(FFT2D_PASS_ROWS, st);
+    if (result != FFT2D_OK)
+        return result;
+    if (!some_rest[0] && !some_rest[1])
+        return some_any[1] ? run_any(FFT2D_PASS_COLS, st) : FFT2D_OK;
+
+    BatchLanes *bl = batch_lanes(device, st);
+    if (!bl)
+        return FFT2D_ERR_OOM;
+    std::unique_lock<std::mutex> lanes_lock(bl->mu);
+    cudaError_t e = batch_lanes_prepare(*bl);
+    if (e == cudaSuccess)
+        e = lanes_wait_stream(*bl, st);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "batch lanes");
+    int group = 0;
+    auto lane = [&] { return bl->s[group++ % kBatchLanes]; };
+    // the groups of one length: a grouped launch, or (lines of 8192 and 16384
+    // points) each image's single-image pass, the same bits
+    auto run_rest = [&](int pass) {
+        const bool row = pass == FFT2D_PASS_ROWS;
+        return batch_groups(
+            n, plans, in, out, row,
+            [&](int L) { return values[pass][L] > 0 && !any[pass][L]; },
+            [&](fft2d::BatchTable &table, int L, int first) {
+                cudaStream_t ls = lane();
+                int *err = plans[first]->dev_err;
+                cudaError_t e = cudaSuccess;
+                if (L < 13) {
+                    e = fft2d::launch_batch_pass(row, L, table, batch_variant(device, pass, L), err,
+                                                 ls);
+                } else {
+                    for (int k = 0; k < table.n && e == cudaSuccess; k++) {
+                        const fft2d::BatchJob &j = table.job[k];
+                        fft2d::PassArgs a;
+                        a.in = j.in;
+                        a.out = j.out;
+                        a.tw = j.tw;
+                        a.rows = row ? j.lines : (1 << L);
+                        a.cols = row ? (1 << L) : j.lines;
+                        a.ld = j.ld;
+                        a.scale = j.scale;
+                        a.nst = L;
+                        a.partial = false;
+                        a.err = err;
+                        e = row ? fft2d::launch_row_pass(L, a, ls) : fft2d::launch_col_pass(L, a, ls);
+                    }
+                }
+                return e == cudaSuccess ? FFT2D_OK : cuda_fail(e, "batched pass");
+            });
+    };
+    if (some_rest[0]) {
+        if (some_any[0])
+            result = run_any(FFT2D_PASS_ROWS, lane());
+        if (result == FFT2D_OK)
+            result = run_rest(FFT2D_PASS_ROWS);
+        if (result == FFT2D_OK && some_rest[1]) {
+            // the column pass starts once every row group has finished
+            e = stream_wait_lanes(*bl, bl->s[0]);
+            if (e == cudaSuccess)
+                e = lanes_wait_stream(*bl, bl->s[0]);
+            if (e != cudaSuccess)
+                result = cuda_fail(e, "batch lanes");
+        }
+    }
+    if (result == FFT2D_OK && some_rest[1]) {
+        if (some_any[1])
+            result = run_any(FFT2D_PASS_COLS, lane());
+        if (result == FFT2D_OK)
+            result = run_rest(FFT2D_PASS_COLS);
+    }
+    // the caller's stream waits for the lanes, after an error too
+    e = stream_wait_lanes(*bl, st);
+    if (e != cudaSuccess && result == FFT2D_OK)
+        result = cuda_fail(e, "batch lanes");
+    if (result == FFT2D_OK && !some_rest[1] && some_any[1])
+        result = run_any(FFT2D_PASS_COLS, st);
+    return result;
+}
+
+// The batch autotuner: every (pass, L, direction) group is launched once per
+// variant and timed on `st`, and the fastest variant per (pass, L) recorded.
+fft2d_status batched_tune(int n, const fft2d_plan_t *plans, const void *const *in,
+                          void *const *out, cudaStream_t st)
+{
+    fft2d::NvtxRange range("fft2d batched autotune");
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (timing && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess))
+    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return cuda_fail(cudaGetLastError(), "cudaEventCreate");
     std::map<std::pair<int, int>, std::vector<float>> times;   // (pass, L) -> ms per variant
     fft2d_status result = FFT2D_OK;
     for (int pass = 0; pass < 2 && result == FFT2D_OK; pass++) {
         const bool row = pass == FFT2D_PASS_ROWS;
-        if (bl && !row) {
-            // the column pass starts once every row group has finished
-            cudaError_t e = stream_wait_lanes(*bl, bl->s[0]);
-            if (e == cudaSuccess)
-                e = lanes_wait_stream(*bl, bl->s[0]);
-            if (e != cudaSuccess) {
-                result = cuda_fail(e, "batch lanes");
-                break;
-            }
-        }
-        for (int L = 1; L <= 14 && result == FFT2D_OK; L++) {
-            for (int dir = -1; dir <= 1 && result == FFT2D_OK; dir += 2) {
-                table.n = 0;
-                int *err = nullptr;
-                int first = -1;
-                for (int i = 0; i <= n; i++) {
-                    const bool flush = (i == n) || table.n == fft2d::kBatchTmaMaxJobs;
-                    if (flush && table.n > 0) {
-                        const int nv = row ? fft2d::kBatchRowVariants : fft2d::kBatchColVariants;
-                        if (!timing && L >= 13) {
-                            // lines of 8192 and 16384 points: each image's
-                            // single-image pass (the cluster column kernels,
-                            // the 5-stage-group rows), the same bits
-                            cudaStream_t ls = bl->s[group++ % kBatchLanes];
-                            cudaError_t e = cudaSuccess;
-                            for (int jj = 0; jj < table.n && e == cudaSuccess; jj++) {
-                                const fft2d::BatchJob &j = table.job[jj];
-                                fft2d::PassArgs a;
-                                a.in = j.in;
-                                a.out = j.out;
-                                a.tw = j.tw;
-                                a.rows = row ? j.lines : (1 << L);
-                                a.cols = row ? (1 << L) : j.lines;
-                                a.ld = j.ld;
-                                a.scale = j.scale;
-                                a.nst = L;
-                                a.partial = false;
-                                a.err = err;
-                                e = row ? fft2d::launch_row_pass(L, a, ls)
-                                        : fft2d::launch_col_pass(L, a, ls);
-                            }
-                            if (e != cudaSuccess) {
-                                result = cuda_fail(e, "batched pass");
-                                break;
-                            }
-                        } else if (!timing) {
-                            const int v = batch_variant(plans[first]->device, pass, L);
-                            cudaStream_t ls = bl->s[group++ % kBatchLanes];
-                            cudaError_t e = fft2d::launch_batch_pass(row, L, table, v, err, ls);
-                            if (e != cudaSuccess) {
-                                result = cuda_fail(e, "batched pass");
-                                break;
-                            }
-                        } else {
-                            auto &tv = times[std::make_pair(pass, L)];
-                            tv.resize(nv, 0.f);
-                            for (int v = 0; v < nv && result == FFT2D_OK; v++) {
-                                cudaError_t e = fft2d::launch_batch_pass(row, L, table, v, err, st);
-                                if (e == cudaSuccess)
-                                    e = cudaEventRecord(e0, st);
-                                for (int r = 0; r < 3 && e == cudaSuccess; r++)
-                                    e = fft2d::launch_batch_pass(row, L, table, v, err, st);
-                                if (e == cudaSuccess)
-                                    e = cudaEventRecord(e1, st);
-                                if (e == cudaSuccess)
-                                    e = cudaEventSynchronize(e1);
-                                float ms = 0.f;
-                                if (e == cudaSuccess)
-                                    e = cudaEventElapsedTime(&ms, e0, e1);
-                                if (e != cudaSuccess)
-                                    result = cuda_fail(e, "batched tuning");
-                                tv[v] += ms;
-                            }
-                        }
-                        table.n = 0;
-                    }
-                    if (i == n)
-                        break;
-                    const fft2d_plan_s *p = plans[i];
-                    if (p->Lr == 0 || p->Lc == 0 || (row ? p->Lc : p->Lr) != L || p->dir != dir)
-                        continue;
-                    if (first < 0) {
-                        first = i;
-                        err = p->dev_err;
-                    }
-                    fft2d::BatchJob &j = table.job[table.n++];
-                    j.in = static_cast<const float2 *>(row ? in[i] : out[i]);
-                    j.out = static_cast<float2 *>(out[i]);
-                    j.tw = row ? p->tw_rows : p->tw_cols;
-                    j.ld = p->cols;
-                    j.lines = row ? p->rows : p->cols;
-                    j.first_cta = 0;
-                    j.scale = (!row && p->dir == FFT2D_INVERSE)
-                                  ? (float)(1.0 / ((double)p->rows * (double)p->cols))
-                                  : 1.0f;
+        result = batch_groups(
+            n, plans, in, out, row, [](int) { return true; },
+            [&](fft2d::BatchTable &table, int L, int first) {
+                const int nv = row ? fft2d::kBatchRowVariants : fft2d::kBatchColVariants;
+                int *err = plans[first]->dev_err;
+                auto &tv = times[std::make_pair(pass, L)];
+                tv.resize(nv, 0.f);
+                for (int v = 0; v < nv; v++) {
+                    cudaError_t e = fft2d::launch_batch_pass(row, L, table, v, err, st);
+                    if (e == cudaSuccess)
+                        e = cudaEventRecord(e0, st);
+                    for (int r = 0; r < 3 && e == cudaSuccess; r++)
+                        e = fft2d::launch_batch_pass(row, L, table, v, err, st);
+                    if (e == cudaSuccess)
+                        e = cudaEventRecord(e1, st);
+                    if (e == cudaSuccess)
+                        e = cudaEventSynchronize(e1);
+                    float ms = 0.f;
+                    if (e == cudaSuccess)
+                        e = cudaEventElapsedTime(&ms, e0, e1);
+                    if (e != cudaSuccess)
+                        return cuda_fail(e, "batched tuning");
+                    tv[v] += ms;
                 }
-            }
+                return FFT2D_OK;
+            });
+    }
+    if (result == FFT2D_OK && n > 0) {
+        std::lock_guard<std::mutex> lock(g_tune_mu);
+        load_tune_file_locked(plans[0]->device);
+        for (auto &kv : times) {
+            const auto &tv = kv.second;
+            int best = 0;
+            for (int v = 1; v < (int)tv.size(); v++)
+                if (tv[v] < tv[best])
+                    best = v;
+            g_tuned[std::make_tuple(plans[0]->device, kv.first.first + 2, kv.first.second, 0)] = best;
         }
+        save_tune_file_locked();
     }
-    if (bl) {
-        cudaError_t e = stream_wait_lanes(*bl, st);
-        if (e != cudaSuccess && result == FFT2D_OK)
-            result = cuda_fail(e, "batch lanes");
-    }
-    if (timing) {
-        if (result == FFT2D_OK && n > 0) {
-            std::lock_guard<std::mutex> lock(g_tune_mu);
-            load_tune_file_locked(plans[0]->device);
-            for (auto &kv : times) {
-                const auto &tv = kv.second;
-                int best = 0;
-                for (int v = 1; v < (int)tv.size(); v++)
-                    if (tv[v] < tv[best])
-                        best = v;
-                g_tuned[std::make_tuple(plans[0]->device, kv.first.first + 2, kv.first.second, 0)] =
-                    best;
-            }
-            save_tune_file_locked();
-        }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
     return result;
 }
 
@@ -1445,7 +1534,7 @@ fft2d_status fft2d_exec_batched(int n, const fft2d_plan_t *plans, const void *co
                 return s;
         }
     }
-    return batched_impl(n, plans, in, out, st, false);
+    return batched_run(n, plans, in, out, st);
 }
 
 int fft2d_batch_variant_count(int pass)
@@ -1496,7 +1585,7 @@ fft2d_status fft2d_autotune_batched(int n, const fft2d_plan_t *plans, const void
     fft2d_status s = batched_check(n, plans, in, out);
     if (s != FFT2D_OK)
         return s;
-    s = batched_impl(n, plans, in, out, static_cast<cudaStream_t>(stream), true);
+    s = batched_tune(n, plans, in, out, static_cast<cudaStream_t>(stream));
     for (int i = 0; i < n; i++)
         cudaMemset(plans[i]->dev_err, 0, sizeof(int));
     return s;

@@ -28,8 +28,9 @@ struct NvtxRange {
 // (CUDA graph) to 1.4 us (stream, host bound) this way, against 2.1 us; a
 // 1024^2 inverse transform takes 10.2 instead of 14.3 us, a 4096^2 forward
 // one 98.8 instead of 103.5, a 4096^2 DCT 65.6 instead of 70.0.  The
-// successor is let in only when this kernel's CTAs have left (no early
-// trigger), so its waiting CTAs never hold room another stream could use.
+// successor is let in only when this kernel's CTAs have left: letting it in
+// early (griddepcontrol.launch_dependents at the start) made nearly every
+// transform slower, 1024^2 9.2 -> 11.1 us and 4096^2 98.6 -> 109.
 // What such a kernel reads through the read-only path, or through a
 // __restrict__ const pointer, may be fetched before the wait: only a plan's
 // tables are read so, never image data, and chained = false is for callers
@@ -190,6 +191,7 @@ struct BatchJob {
     int lines;       // rows (row pass) or columns (column pass) of the image
     int first_cta;   // filled by launch_batch_pass
     float scale;
+    int L;           // log2 of the line length (launch_batch_any)
 };
 struct BatchTable {
     int n;
@@ -231,6 +233,7 @@ struct BatchJobH16 {
     int lines;           // rows (row pass) or columns (column pass) of the image
     int first_cta;       // filled by launch_batch_pass_h16
     float scale;
+    int L;               // log2 of the line length (launch_batch_any_h16)
 };
 struct BatchTableH16 {
     int n;
@@ -255,6 +258,31 @@ const char *batch_variant_name(bool row, int variant);
 // to the plain grouped kernel.
 cudaError_t launch_batch_pass(bool row, int L, BatchTable &t, int variant, int *err,
                               cudaStream_t s);
+
+// One launch for jobs of any axis lengths (batch_any.cu): the tiles of 2^12
+// values (256 threads x 16), each CTA with its job's length and rotation
+// factors.  Lengths 2^1 .. 2^kBatchAnyMaxL.
+constexpr int kBatchAnyMaxL = 12;
+cudaError_t launch_batch_any(bool row, BatchTable &t, cudaStream_t s);
+cudaError_t launch_batch_any_h16(bool row, BatchTableH16 &t, int in_axis, cudaStream_t s);
+
+// Whether a group of one axis length (`values` over all its images) joins the
+// launch for any length, in a batch of `total` values.  Batches of up to 2^23
+// values only: above, the launches are not what counts, and one kernel with
+// every length's code loses to a kernel per length (64 images of 128 .. 2048,
+// 55 M values: 351 against 337 us).  Below: 16 images of 64 .. 128 (0.2 M) 19.9
+// against 33.2 us a call, 10.4 / 13.6 replayed from a graph; 64 images of 128
+// .. 512 (5.8 M) 60 / 84 and 43 / 49; 32 images of 128 .. 1024 (8.5 M) even.
+// Rows run the CTAs of their own kernels.  Columns of up to 512 rows join, and
+// longer ones as long as the group fits 128 CTAs of 2^12 values
+// (col_small_tile): beyond that their 32-byte row segments lose to the wider
+// tiles of their own kernels.
+constexpr long long kBatchAnyTotal = 1ll << 23;
+constexpr bool batch_any(bool row, int L, long long values, long long total)
+{
+    return total <= kBatchAnyTotal && L <= kBatchAnyMaxL &&
+           (row || L <= 9 || (L <= 11 && col_small_tile(values) == 12));
+}
 
 // 3D tensor map over a column-pass image of 8-byte elements (rows a
 // multiple of 256): x = column, y = row within a block of 256 rows, z =

@@ -123,16 +123,27 @@ cudaError_t h16_phase(const std::vector<Req *> &reqs, const std::vector<fft2d_pl
         if (e != cudaSuccess)
             return e;
     }
-    // the rest: row groups by row length, then column groups by column length
+    // the rest: per pass one launch for any axis length where that serves the
+    // length, then a launch per other length
     for (int pass = 0; pass < 2; pass++) {
         const bool row = pass == 0;
-        for (int L = 1; L <= 14; L++) {
+        const int axis = row ? in_axis : 0;
+        long long values[15] = {}, total = 0;
+        for (size_t i = 0; i < n; i++)
+            if (grouped(i)) {
+                values[row ? pv[i].Lc : pv[i].Lr] += (long long)pv[i].rows * pv[i].cols;
+                total += (long long)pv[i].rows * pv[i].cols;
+            }
+        for (int want = 0; want <= 14; want++) {   // 0: the launch for any length
+            if (want > 0 && (values[want] == 0 || fft2d::batch_any(row, want, values[want], total)))
+                continue;
             table.n = 0;
             for (size_t i = 0; i <= n; i++) {
                 const bool flush = i == n || table.n == fft2d::kBatchH16MaxJobs;
                 if (flush && table.n > 0) {
-                    cudaError_t e = fft2d::launch_batch_pass_h16(row, L, table,
-                                                                 row ? in_axis : 0, st);
+                    cudaError_t e = want == 0
+                                        ? fft2d::launch_batch_any_h16(row, table, axis, st)
+                                        : fft2d::launch_batch_pass_h16(row, want, table, axis, st);
                     if (e != cudaSuccess)
                         return e;
                     table.n = 0;
@@ -140,7 +151,9 @@ cudaError_t h16_phase(const std::vector<Req *> &reqs, const std::vector<fft2d_pl
                 if (i == n)
                     break;
                 const fft2d::PlanView &v = pv[i];
-                if (!grouped(i) || (row ? v.Lc : v.Lr) != L)
+                const int L = row ? v.Lc : v.Lr;
+                if (!grouped(i) ||
+                    (want == 0 ? !fft2d::batch_any(row, L, values[L], total) : L != want))
                     continue;
                 const Req *q = reqs[i];
                 fft2d::BatchJobH16 &j = table.job[table.n++];
@@ -155,6 +168,7 @@ cudaError_t h16_phase(const std::vector<Req *> &reqs, const std::vector<fft2d_pl
                 j.scale = (!row && v.dir == FFT2D_INVERSE)
                               ? (float)(1.0 / ((double)v.rows * (double)v.cols))
                               : 1.0f;
+                j.L = L;
             }
         }
     }

@@ -15,14 +15,13 @@
 // takes 5.0 us against 10.1 in two launches.  Why 4096 values per CTA: the same 64-register,
 // 32 KB configuration serves every axis from 2 to 4096 points, and 16 CTAs
 // spread 2^16 pixels over as many SMs as one cluster may span.
-#include "line_fft.cuh"
+#include "any_axis.cuh"
 #include "passes.h"
 
 namespace fft2d {
 
 namespace {
 
-constexpr int kSmallL = 12;               // log2 of the values per CTA
 constexpr int kSmallMaxCtas = 16;         // largest cluster (non-portable above 8)
 
 // The column phase reads what other CTAs of the cluster have just written.
@@ -34,37 +33,6 @@ struct StoreH16Shared : StoreH16T<IA> {
     static constexpr bool CG = true;
 };
 
-template <int L, bool ROW, class IO>
-__device__ __forceinline__ void small_axis(const IO &io, const float2 *__restrict__ tw, float scale,
-                                           int cta, int lines, int ld)
-{
-    using C = LineCfg<L, ROW ? 0 : kSmallL - L, ROW ? kSmallL - L : 0>;
-    constexpr int PER = 1 << (kSmallL - L);   // lines per CTA
-    const long long l0 = (long long)cta * PER;
-    line_fft<C, ROW, true, IO>(io, ROW ? Geo{l0, 1, 0, ld} : Geo{0, 1, l0, ld}, tw, scale, L,
-                               lines - l0);
-}
-
-template <bool ROW, class IO>
-__device__ __forceinline__ void small_phase(int L, const IO &io, const float2 *__restrict__ tw,
-                                            float scale, int cta, int lines, int ld)
-{
-    switch (L) {
-    case 1: return small_axis<1, ROW>(io, tw, scale, cta, lines, ld);
-    case 2: return small_axis<2, ROW>(io, tw, scale, cta, lines, ld);
-    case 3: return small_axis<3, ROW>(io, tw, scale, cta, lines, ld);
-    case 4: return small_axis<4, ROW>(io, tw, scale, cta, lines, ld);
-    case 5: return small_axis<5, ROW>(io, tw, scale, cta, lines, ld);
-    case 6: return small_axis<6, ROW>(io, tw, scale, cta, lines, ld);
-    case 7: return small_axis<7, ROW>(io, tw, scale, cta, lines, ld);
-    case 8: return small_axis<8, ROW>(io, tw, scale, cta, lines, ld);
-    case 9: return small_axis<9, ROW>(io, tw, scale, cta, lines, ld);
-    case 10: return small_axis<10, ROW>(io, tw, scale, cta, lines, ld);
-    case 11: return small_axis<11, ROW>(io, tw, scale, cta, lines, ld);
-    case 12: return small_axis<12, ROW>(io, tw, scale, cta, lines, ld);
-    }
-}
-
 // One cluster = the whole grid.  rio / cio: the storage of the two phases.
 template <class RIO, class CIO>
 __global__ void __launch_bounds__(256, 4) small_kernel(const RIO rio, const CIO cio,
@@ -73,24 +41,19 @@ __global__ void __launch_bounds__(256, 4) small_kernel(const RIO rio, const CIO 
                                                        int cols, int Lr, int Lc, float scale)
 {
     const int cta = (int)blockIdx.x;
-    small_phase<true>(Lc, rio, tw_rows, 1.0f, cta, rows, cols);
+    any_axis<true>(Lc, rio, tw_rows, 1.0f, cta, rows, cols);
     // every row is in `out` before any column is read, and the exchange
     // buffer is free again
     asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                  "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    small_phase<false>(Lr, cio, tw_cols, scale, cta, cols, cols);
+    any_axis<false>(Lr, cio, tw_cols, scale, cta, cols, cols);
 }
-
-// Exchange buffer of 2^12 values, or (axes of up to 16 points: no exchange)
-// the half2 exponent reduction of up to 2^11 lines; with an exchange, at most
-// 2^7 lines reduce behind it.
-constexpr int kSmallSmem = (1 << kSmallL) * 8 + 128 * 4;
 
 template <class RIO, class CIO>
 cudaError_t small_launch(const RIO &rio, const CIO &cio, const SmallArgs &a, cudaStream_t s)
 {
     auto k = small_kernel<RIO, CIO>;
-    const int ctas = a.Lr + a.Lc > kSmallL ? 1 << (a.Lr + a.Lc - kSmallL) : 1;
+    const int ctas = a.Lr + a.Lc > kAnyL ? 1 << (a.Lr + a.Lc - kAnyL) : 1;
     if (ctas > 8) {
         // clusters above 8 CTAs are opt-in, and a device may refuse them
         static DeviceCache ok;   // 1: usable, 2: not
@@ -107,7 +70,7 @@ cudaError_t small_launch(const RIO &rio, const CIO &cio, const SmallArgs &a, cud
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3(kSmallMaxCtas);
                 cfg.blockDim = dim3(256);
-                cfg.dynamicSmemBytes = kSmallSmem;
+                cfg.dynamicSmemBytes = kAnySmem;
                 cfg.attrs = at;
                 cfg.numAttrs = 1;
                 e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
@@ -119,7 +82,7 @@ cudaError_t small_launch(const RIO &rio, const CIO &cio, const SmallArgs &a, cud
         if (ok.get(d) != 1)
             return cudaErrorNotSupported;
     }
-    return launch_chained(k, dim3(ctas), 256, kSmallSmem, s, LaunchHow((unsigned)ctas), rio, cio,
+    return launch_chained(k, dim3(ctas), 256, kAnySmem, s, LaunchHow((unsigned)ctas), rio, cio,
                           a.tw_rows, a.tw_cols, 1 << a.Lr, 1 << a.Lc, a.Lr, a.Lc, a.scale);
 }
 
@@ -128,7 +91,7 @@ cudaError_t small_launch(const RIO &rio, const CIO &cio, const SmallArgs &a, cud
 // 2^16 pixels is the most that one cluster holds at 4096 values per CTA.
 bool small_image(int Lr, int Lc)
 {
-    return Lr >= 1 && Lc >= 1 && Lr <= kSmallL && Lc <= kSmallL && Lr + Lc <= kSmallL + 4;
+    return Lr >= 1 && Lc >= 1 && Lr <= kAnyL && Lc <= kAnyL && Lr + Lc <= kAnyL + 4;
 }
 
 cudaError_t launch_small(const SmallArgs &a, const float2 *in, float2 *out, cudaStream_t s)
