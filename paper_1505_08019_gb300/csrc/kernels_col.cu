@@ -387,6 +387,8 @@ struct ColVariants {
     using Narrow = LineCfg<L, (KWN >= 0 ? KWN : 0), 0>;
     using Fine = LineCfg<L, (L <= 12 ? 12 - L : 0), 0>;
     using Fine5 = LineCfg<9, 3, 0, 32, 5>;
+    using Quarter = LineCfg<10, 2, 0, 32, 5>;
+    using Half = LineCfg<10, 3, 0, 64, 6>;
     // cluster shapes: W = 8 over 2 (2048 rows) or 4 (4096 rows) CTAs;
     // W = 4 over 2 or 4 CTAs for 8192 and 16384 rows
     static constexpr int CKW = L <= 12 ? 3 : 2;
@@ -398,7 +400,7 @@ struct ColVariants {
     using Clu8 = ClusterColCfg<(L >= 13 ? L : 13), 3, (L >= 13 ? L - 11 : 2)>;
 
     struct Table {
-        Variant v[12];
+        Variant v[16];
         int n = 0;
     };
     static Table build()
@@ -462,11 +464,20 @@ struct ColVariants {
             t.v[t.n++] = {"quadl2", PairLocal6::W, 64, col_group_usable<PairLocal6, 2>,
                           col_launch_group_l2<PairLocal6, 2>, true};
         // 4096 values (256 threads) per CTA, for images of few columns
-        if constexpr (L == 10 || L == 11)
+        if constexpr (L == 11)
             t.v[t.n++] = {"fine", Fine::W, 16, whole_stages, col_launch_any<Fine>};
         // 512 rows in two groups (5 + 4), 128 threads x 32 values
         if constexpr (L == 9)
             t.v[t.n++] = {"fine32g5", Fine5::W, 32, whole_stages, col_launch_any<Fine5>};
+        // 1024 rows, TMA-fed with several CTAs per SM: two groups of 5 stages
+        // in 4-column tiles (four CTAs of 128 threads x 32 values), 6 + 4
+        // stages in 8-column tiles (two of 128 x 64)
+        if constexpr (L == 10) {
+            t.v[t.n++] = {"tma32g5", Quarter::W, 32, col_tma_usable<Quarter>,
+                          col_launch_tma<Quarter, false>, true};
+            t.v[t.n++] = {"tma64w8", Half::W, 64, col_tma_usable<Half>,
+                          col_launch_tma<Half, false>, true};
+        }
         // two phases per 32-column strip, the intermediate in L2
         if constexpr (L >= 13)
             t.v[t.n++] = {"stripl2", 32, 16, col_strip_usable, col_launch_strip<L>};
@@ -494,8 +505,11 @@ struct ColVariants {
     // and 3.0 / 4.2 for "plain" up to 2048 columns.  512 rows: "fine32g5"
     // at every width, 2.9 / 3.5 us for "narrow" up to 1024 columns, 13.6 / 15.7
     // at 8192: one exchange instead of two.  1024
-    // rows: "fine" for up to 128 of its CTAs (512 columns), 3.8 against 4.9 us
-    // for "narrow", which wins from 1024 columns (5.2 / 5.5).  2048 rows:
+    // rows: "tma32g5", 3.3 against 4.9 us for "narrow" up to 512 columns, 8.9 /
+    // 9.3 at 2048, 14.8 / 18.2 at 4096, 26.9 / 32.1 at 8192 (four CTAs per SM,
+    // each with the next tile's first half on its way, against two that load,
+    // work and store in turn); above, "tma64w8", 48.4 against 51.5 and 61.1.
+    // 2048 rows:
     // "fine" up to 128 CTAs (256 columns), 5.3 us, "narrow" up to 128 (512
     // columns), 6.0, against 8.1 - 8.5 for the TMA pass in two groups of 6
     // stages with per-thread stores ("tma64st"), which wins from 1024 columns
@@ -515,7 +529,7 @@ struct ColVariants {
         else if constexpr (L == 9)
             return index_of("fine32g5");
         else if constexpr (L == 10)
-            return index_of(cols <= 128 * Fine::W ? "fine" : "narrow");
+            return index_of(cols <= 8192 ? "tma32g5" : "tma64w8");
         else if constexpr (L == 11)
             return index_of(cols <= 128 * Fine::W     ? "fine"
                             : cols <= 128 * Narrow::W ? "narrow"
@@ -599,6 +613,8 @@ int col_selftest_variant(int L, const PassArgs &a)
 {
     if (a.variant >= 0)
         return a.variant;
+    if (L == 10)
+        return ColVariants<10>::index_of("narrow");   // refused, as it always was
     if (L == 11)
         return ColVariants<11>::index_of("tma64st");
     if (L == 13)
