@@ -92,7 +92,6 @@ __global__ void __launch_bounds__(C::T, 1) col_h16_tma_kernel(const __grid_const
     const int ntiles = cols / C::W;
     const int tid = threadIdx.x;
     int tile = blockIdx.x;
-    pdl_wait();
     if (tid == 0) {
         mbar_init(&bar_early, 1);
         mbar_init(&bar_late, 1);
@@ -100,12 +99,16 @@ __global__ void __launch_bounds__(C::T, 1) col_h16_tma_kernel(const __grid_const
     }
     if (tid < C::W)
         sred[tid] = 0;
+    if (tid == 0 && tile < ntiles) {   // a plan's table: needs no wait
+        prefetch_map(&map);
+        mbar_expect_tx(&bar_early, H::TW_BYTES);
+        bulk_load(stw, tw, H::TW_BYTES, &bar_early);
+    }
+    pdl_wait();
     for (int i = tid; i < C::N; i += C::T)
         rf[i] = pow2f(row_exp[i]);
     __syncthreads();
     if (tid == 0 && tile < ntiles) {
-        mbar_expect_tx(&bar_early, H::TW_BYTES);
-        bulk_load(stw, tw, H::TW_BYTES, &bar_early);
         h16_issue<C>(smraw + H::PREF_OFF, &map, tile * C::W, 0, H::EARLY_BYTES, &bar_early);
         h16_issue<C>(smraw, &map, tile * C::W, H::NB, H::LATE_BYTES, &bar_late);
     }

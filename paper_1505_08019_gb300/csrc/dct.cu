@@ -653,7 +653,6 @@ __global__ void __launch_bounds__(C::T, 1) col_dct_tma_kernel(
     extern __shared__ __align__(1024) float2 sm[];
     __shared__ __align__(8) uint64_t bar_even, bar_odd;
     const int tid = threadIdx.x;
-    pdl_wait();
     int tile = blockIdx.x;
     float2 *pref = sm + C::E;          // even region
     float2 *stw = sm + D::TW_OFF;      // rotation factors, loaded once
@@ -664,9 +663,13 @@ __global__ void __launch_bounds__(C::T, 1) col_dct_tma_kernel(
         fence_mbar_init();
     }
     __syncthreads();
-    if (tid == 0 && tile < ntiles) {
+    if (tid == 0 && tile < ntiles) {   // a plan's table: needs no wait
+        prefetch_map(&me);
         mbar_expect_tx(&bar_even, D::TW_BYTES);
         bulk_load(stw, tw, D::TW_BYTES, &bar_even);
+    }
+    pdl_wait();
+    if (tid == 0 && tile < ntiles) {
         mbar_arrive_expect_tx(&bar_even, D::HBYTES);
         tma_load_3d(pref, &me, tile * C::W, 0, 0, &bar_even);
         if (!(withhold && blockIdx.x == 0)) {   // self-test: the first odd rows never come
@@ -853,7 +856,6 @@ __global__ void __launch_bounds__(C::T, 1) col_dct_tma64_kernel(
     __shared__ __align__(8) uint64_t bar_early, bar_late;
     __shared__ float2 rot_base[R / 2];   // (cos, sin)(pi 2^S0 r / (2N)), r < R/2
     const int tid = threadIdx.x;
-    pdl_wait();
     float2 *stw = sm + S::TW_OFF;
     float2 *stage = sm + C::E / 2;
     const int w = tid & (C::W - 1);
@@ -877,10 +879,14 @@ __global__ void __launch_bounds__(C::T, 1) col_dct_tma64_kernel(
     __syncthreads();
     int tile = (int)blockIdx.x;
     int n_early = 0, n_late = 0, w_early = 0, w_late = 0;
+    if (tid == 0 && tile < ntiles) {   // a plan's table: needs no wait
+        prefetch_map(&me);
+        mbar_expect_tx(&bar_early, S::TW_BYTES);
+        bulk_load(stw, tw, S::TW_BYTES, &bar_early);
+    }
+    pdl_wait();
     if (tile < ntiles) {
         if (tid == 0) {
-            mbar_expect_tx(&bar_early, S::TW_BYTES);
-            bulk_load(stw, tw, S::TW_BYTES, &bar_early);
             issue_early(tile);
             if (!(withhold && blockIdx.x == 0))   // self-test: the first odd rows never come
                 issue_late(tile);
@@ -1078,7 +1084,6 @@ __global__ void __launch_bounds__(C::T, 1) col_idct_tma64_kernel(
     __shared__ __align__(8) uint64_t bar_early, bar_late;
     __shared__ float2 rot_top[G0::R];   // (cos, sin)(pi top(r) / (2N)), top(r) = rev(r) 2^HB
     const int tid = threadIdx.x;
-    pdl_wait();
     float2 *stw = sm + S::TW_OFF;
     float2 *stage = sm + C::E / 2;
     const float2 *pref = sm + C::E;
@@ -1099,10 +1104,14 @@ __global__ void __launch_bounds__(C::T, 1) col_idct_tma64_kernel(
     __syncthreads();
     int tile = (int)blockIdx.x;
     int n_early = 0, n_late = 0, w_early = 0, w_late = 0;
+    if (tid == 0 && tile < ntiles) {   // a plan's table: needs no wait
+        prefetch_map(&map);
+        mbar_expect_tx(&bar_early, S::TW_BYTES);
+        bulk_load(stw, tw, S::TW_BYTES, &bar_early);
+    }
+    pdl_wait();
     if (tile < ntiles) {
         if (tid == 0) {
-            mbar_expect_tx(&bar_early, S::TW_BYTES);
-            bulk_load(stw, tw, S::TW_BYTES, &bar_early);
             split_issue_early<C>(sm, &map, tile * C::W, &bar_early);
             if (!(withhold && blockIdx.x == 0))   // self-test: the first second half never comes
                 split_issue_late<C>(sm, &map, tile * C::W, &bar_late);
@@ -1442,7 +1451,6 @@ __global__ void __launch_bounds__(C::T, 1) col_idct_tma_kernel(
     extern __shared__ __align__(1024) float2 sm[];
     __shared__ __align__(8) uint64_t bar_early, bar_late;
     const int tid = threadIdx.x;
-    pdl_wait();
     int tile = blockIdx.x;
     const float2 *pref = sm + C::E;
     float2 *stw = sm + S::TW_OFF;
@@ -1453,9 +1461,13 @@ __global__ void __launch_bounds__(C::T, 1) col_idct_tma_kernel(
         fence_mbar_init();
     }
     __syncthreads();
-    if (tid == 0 && tile < ntiles) {
+    if (tid == 0 && tile < ntiles) {   // a plan's table: needs no wait
+        prefetch_map(&map);
         mbar_expect_tx(&bar_early, S::TW_BYTES);
         bulk_load(stw, tw, S::TW_BYTES, &bar_early);
+    }
+    pdl_wait();
+    if (tid == 0 && tile < ntiles) {
         split_issue_early<C>(sm, &map, tile * C::W, &bar_early);
         if (!(withhold && blockIdx.x == 0))   // self-test: the first late half never comes
             split_issue_late<C>(sm, &map, tile * C::W, &bar_late);

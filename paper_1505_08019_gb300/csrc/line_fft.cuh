@@ -1110,13 +1110,18 @@ __device__ __forceinline__ void col_tma2_body(const Src &src, int ntiles,
         fence_mbar_init();
     }
     __syncthreads();
-    pdl_wait();
     // the rotation factors (N entries, the last one padding) stay in shared
-    // memory for the CTA's whole life; they arrive with the first tile
+    // memory for the CTA's whole life; they are a plan's (or noalloc's, whose
+    // passes are not chained), so their load need not wait for the previous
+    // kernel as the image's must (4096^2 transform 98.6 -> 98.0 us)
     float2 *stw = sm + TmaSplit<C>::TW_OFF;
     if (tid == 0 && tile < ntiles) {
+        prefetch_map(src.tmap(tile));
         mbar_expect_tx(&bar_early, TmaSplit<C>::TW_BYTES);
         bulk_load(stw, tw, TmaSplit<C>::TW_BYTES, &bar_early);
+    }
+    pdl_wait();
+    if (tid == 0 && tile < ntiles) {
         split_issue_early<C>(sm, src.tmap(tile), src.col(tile), &bar_early);
         if (!(withhold && blockIdx.x == 0))
             split_issue_late<C>(sm, src.tmap(tile), src.col(tile), &bar_late);
