@@ -1,10 +1,8 @@
 // col_h16.cuh -- persistent TMA-fed column pass for half2 storage (one
 // power-of-two exponent per line, FP32 arithmetic).
 //
-// The arithmetic is the FP32 column engine's (a tile of W = 4 whole columns
-// of 2^L rows; 256 threads x 64 values in two groups of radix-2 DIT stages,
-// or 512 x 32 in three,
-// Section 2 eqs. 2-3 / Section 3.1 eq. 4, the scramble of Section 3.2 fused
+// The arithmetic is the FP32 column engine's (a tile of W = 4 or 8 whole
+// columns of 2^L rows in two groups of radix-2 DIT stages, Section 2 eqs. 2-3 / Section 3.1 eq. 4, the scramble of Section 3.2 fused
 // into the first read), so the results are those of the complex64 column
 // pass on the dequantised input, rounded once to half precision at the end.
 // Only the storage differs:
@@ -12,7 +10,7 @@
 //  * The tile arrives as half2 (4 bytes a pixel): its first half (the early
 //    256-row blocks) in a prefetch region, its second half at the start of
 //    the FP32 exchange region once the previous tile's last group has read
-//    it, both by TMA with 16-byte box rows.
+//    it, both by TMA with 16- or 32-byte box rows.
 //  * Group 0 gathers it scrambled, widens each value to FP32 and applies its
 //    row's input scale 2^e (the row pass's exponents, converted once per CTA
 //    into a table of factors in shared memory).
@@ -47,10 +45,7 @@ struct H16Col {
     static constexpr int RF_OFF = TW_OFF + (int)TW_BYTES;         // 2^e of every image row
     static constexpr int SMEM_BYTES = RF_OFF + C::N * 4;
     static constexpr int STAGE_OFF = X_BYTES / 2;           // finished half2 tile
-    static_assert(C::W == 4 && C::LB == 1 &&
-                      ((C::EPT == 32 && C::NG == 3) || (C::EPT == 64 && C::NG == 2)),
-                  "4-column tiles; 512 threads x 32 values in three stage groups or 256 x 64 "
-                  "in two");
+    static_assert((C::W == 4 || C::W == 8) && C::LB == 1 && C::NG >= 2, "4- or 8-column tiles");
     static_assert(NB >= 1 && 2 * NB == NBOX, "two equal halves of whole blocks");
     static_assert(LATE_BYTES <= (uint32_t)STAGE_OFF, "the late half and the staging never overlap");
     static_assert(STAGE_OFF + C::E * 4 <= X_BYTES, "the staging fits in the exchange region");

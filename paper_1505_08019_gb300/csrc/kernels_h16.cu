@@ -69,16 +69,15 @@ bool encode_h16_col_map(CUtensorMap *map, const __half2 *base, int rows, int col
            CUDA_SUCCESS;
 }
 
-// The persistent TMA-fed half2 column pass (col_h16.cuh) for columns of
-// 2^L rows in 4-column tiles.  Returns cudaErrorNotSupported (nothing
-// launched) when the buffers or shape cannot feed it: the caller then takes
-// another kernel.
-template <int L>
+// The persistent TMA-fed half2 column pass (col_h16.cuh) with tiles of C, as
+// many CTAs per SM as fit.  Returns cudaErrorNotSupported (nothing launched)
+// when the buffers or shape cannot feed it: the caller then takes another
+// kernel.
+template <class C>
 cudaError_t h16_launch_col_tma(const H16PassArgs &a, cudaStream_t s)
 {
-    using C = LineCfg<L, 2, 0, 64, 6>;   // two groups of 6 stages, as the complex64 pass
     using H = H16Col<C>;
-    if (a.in_axis != 0 || a.nst != L || !a.err || a.cols % C::W != 0 ||
+    if (a.in_axis != 0 || a.nst != C::L || !a.err || a.cols % C::W != 0 ||
         (reinterpret_cast<uintptr_t>(a.tw) & 15))
         return cudaErrorNotSupported;
     CUtensorMap map, omap;
@@ -86,17 +85,21 @@ cudaError_t h16_launch_col_tma(const H16PassArgs &a, cudaStream_t s)
         !encode_h16_col_map(&omap, a.out, a.rows, a.cols, a.ld, C::W, H::BOX, H::NBOX))
         return cudaErrorNotSupported;
     auto k = col_h16_tma_kernel<C>;
-    static DeviceCache ready;
+    static DeviceCache occ;
     const int d = device_current();
-    if (!ready.get(d)) {
+    if (!occ.get(d)) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              H::SMEM_BYTES);
         if (e != cudaSuccess)
             return e;
-        ready.set(d, 1);
+        int o = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, C::T, H::SMEM_BYTES);
+        if (e != cudaSuccess)
+            return e;
+        occ.set(d, o > 0 ? o : 1);
     }
     const int ntiles = a.cols / C::W;
-    int grid = device_sm_count();
+    int grid = device_sm_count() * occ.get(d);
     if (grid > ntiles)
         grid = ntiles;
     return launch_chained(k, (unsigned)grid, C::T, H::SMEM_BYTES, s, 1, map, omap, a.tw, a.in_exp,
@@ -204,8 +207,31 @@ cudaError_t h16_dispatch(bool row, const H16PassArgs &a, cudaStream_t s)
         if (tile == 13)
             return h16_launch_col_tile<LineCfg<L, 13 - L, 0>>(a, s);
     }
+    if constexpr (L >= 9 && L <= 11) {
+        // many columns (2^22 values): the TMA-fed pass, 512 rows in 8-column
+        // tiles of 128 threads x 32 values, 1024 rows the same in 4-column
+        // ones (up to 8192 columns; above in 8-column tiles of 128 x 64), 2048
+        // rows in 8-column tiles of 256 x 64.  Whole transform, plain column
+        // pass and here: 512x16384 59.7 / 54.2 us, 1024x4096 29.3 / 28.0,
+        // 1024x8192 59.0 / 49.8, 1024x16384 119 / 104, 2048x2048 32.6 / 29.5,
+        // 2048x4096 61.3 / 49.7, 2048x16384 263 / 201.  Below the line the
+        // plain kernel's shorter start wins (1024x2048 15.8 / 17.8).
+        if ((long long)a.cols << L >= 1ll << 22) {
+            using Wide = typename std::conditional<
+                L == 9, LineCfg<9, 3, 0, 32, 5>,
+                typename std::conditional<L == 10, LineCfg<10, 2, 0, 32, 5>,
+                                          LineCfg<11, 3, 0, 64, 6>>::type>::type;
+            using Widest =
+                typename std::conditional<L == 10, LineCfg<10, 3, 0, 64, 6>, Wide>::type;
+            const cudaError_t e = a.cols <= 8192 ? h16_launch_col_tma<Wide>(a, s)
+                                                 : h16_launch_col_tma<Widest>(a, s);
+            if (e != cudaErrorNotSupported)
+                return e;
+        }
+    }
     if constexpr (L == 12) {
-        const cudaError_t e = h16_launch_col_tma<L>(a, s);
+        // two groups of 6 stages, as the complex64 pass
+        const cudaError_t e = h16_launch_col_tma<LineCfg<12, 2, 0, 64, 6>>(a, s);
         if (e != cudaErrorNotSupported)
             return e;
     }

@@ -50,7 +50,11 @@ def test_column_tiles_dct(rows, cols, inverse):
         assert torch.equal(x, out)
 
 
-@pytest.mark.parametrize("rows,cols", [(r, c) for r, c in CASES if r > 64])
+# the half2 TMA line: 2^22 values, and above 8192 columns
+HALF_WIDE = [(512, 4096), (512, 8192), (512, 16384), (1024, 8192), (1024, 16384), (2048, 4096)]
+
+
+@pytest.mark.parametrize("rows,cols", [(r, c) for r, c in CASES if r > 64] + HALF_WIDE)
 def test_column_tiles_half(rows, cols):
     """Whole half2 transform against 64 bits within the half2 tests' 5e-3, and
     the stored range of every column."""
