@@ -46,6 +46,28 @@ __device__ __forceinline__ float2 ld_img(const float2 *p)
     return v;
 }
 
+// Loads through L2 only, for data that other CTAs wrote during this kernel (or
+// the previous one): volatile, so that they stay behind the barrier or wait
+// that orders them (__ldcg need not).
+__device__ __forceinline__ float ld_l2(const float *p)
+{
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_l2(const float2 *p)
+{
+    float2 v;
+    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int ld_l2(const int *p)
+{
+    int v;
+    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ uint32_t smem_addr(const void *p)
 {
     return (uint32_t)__cvta_generic_to_shared(p);

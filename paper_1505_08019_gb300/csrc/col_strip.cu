@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(256, 4) col_strip_kernel(const StripArgs g)
             for (int j = 0; j < 16; j++) {
                 const int set = LB == 7 ? u >> 3 : j / 8;
                 const int b = LB == 7 ? j | (u & 7) << 4 : j % 8 | u << 3;
-                a[j] = __ldcg(slot + ((b << LA) | (set ? lo1 : lo0)) * kStripCols + wb);
+                a[j] = ld_l2(slot + ((b << LA) | (set ? lo1 : lo0)) * kStripCols + wb);
             }
             if (tid < 2 * (NB - 1)) {
                 const int set = tid / (NB - 1), e = tid % (NB - 1) + 1;

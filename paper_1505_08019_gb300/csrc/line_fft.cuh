@@ -295,7 +295,7 @@ __device__ __forceinline__ float in_factor(const IO &io, const Geo &g, int lb, i
     const long long line = io.axis() == 0 ? (ROW ? g.r0 + lb : g.r0 + (long long)i * g.rstep)
                                           : (ROW ? (long long)i : g.c0 + w);
     if constexpr (IO::CG)
-        return pow2f(__ldcg(io.in_exp + line));
+        return pow2f(ld_l2(io.in_exp + line));
     return pow2f(io.in_exp[line]);
 }
 
@@ -310,16 +310,18 @@ __device__ __forceinline__ float2 load_pix(const IO &io, const Geo &g, int lb, i
     } else if constexpr (IO::H16) {
         const long long k = pix<ROW>(g, lb, i, w);
         __half2 h;
-        if constexpr (IO::CG)
-            h = __ldcg(io.in + k);
-        else
+        if constexpr (IO::CG) {
+            const int bits = ld_l2(reinterpret_cast<const int *>(io.in + k));
+            h = *reinterpret_cast<const __half2 *>(&bits);
+        } else {
             h = io.in[k];
+        }
         const float2 q = __half22float2(h);
         if constexpr (!H16PerUnit<IO, ROW>::value)
             f = in_factor<IO, ROW>(io, g, lb, i, w);
         return make_float2(q.x * f, q.y * f);
     } else if constexpr (IO::CG) {
-        return __ldcg(io.in + pix<ROW>(g, lb, i, w));
+        return ld_l2(io.in + pix<ROW>(g, lb, i, w));
     } else {
         return ld_stream(io.in + pix<ROW>(g, lb, i, w));
     }
