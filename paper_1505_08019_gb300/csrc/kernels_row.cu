@@ -2,7 +2,7 @@
 // line of cols = 2^L contiguous points.
 //
 // Variants per line length (the autotuner picks among the usable ones):
-//   0  plain   : LB = 2^row_kb(L) rows per CTA, 256 threads x 16 values,
+//   0  plain   : LB = 2^row_kb(L) rows per CTA, 16 values per thread,
 //                scrambled global loads (the default)
 //   1  plain32 : the same rows per CTA with 32 values per thread
 //   2  plain2x : twice the rows per CTA (two line blocks in flight)

@@ -109,11 +109,20 @@ const Variant *col_variants(int L, int *n);
 int row_default_variant(int L);
 int col_default_variant(int L, int cols);
 
-// Per-size CTA shapes of the plain kernels: log2 of the rows per CTA of the
-// row pass (256 threads per CTA up to 4096-point rows) and log2 of the
-// adjacent columns per CTA of the column pass (2^14 values per CTA from
-// 1024-point columns up, 16 to 64 columns below).
-constexpr int row_kb(int L) { return L <= 12 ? 12 - L : 0; }
+// Per-size CTA shapes of the plain kernels.  Row pass, log2 of the rows per
+// CTA: 2^9 values up to 16-point rows, 2^10 up to 64, 2^11 up to 2048, one row
+// above -- 16 values a thread, so 32 to 128 threads, which spread few or short
+// rows over more SMs and start and end faster.  Measured against 2^12 values
+// throughout (complex64 / forward / inverse DCT, us): 1024x16 5.1 / 9.5 / 9.4 ->
+// 2.7 / 2.7 / 2.6, 2048x32 3.7 / 6.2 / 7.0 -> 2.6 / 3.5 / 2.9, 2048x128 3.1 / 4.9 /
+// 4.5 -> 2.7 / 3.7 / 2.9, 2048x1024 6.5 / 5.6 / 5.1 -> 5.8 / 5.3 / 4.8, 8192x2048
+// 43.9 / 28.0 / 30.5 -> 42.5 / 28.5 / 29.2.  Column pass, log2 of the adjacent
+// columns per CTA (2^14 values per CTA from 1024-point columns up, 16 to 64
+// columns below).
+constexpr int row_kb(int L)
+{
+    return L <= 4 ? 9 - L : L <= 6 ? 10 - L : L <= 11 ? 11 - L : 0;
+}
 constexpr int col_kw(int L)
 {
     return L >= 10 ? 14 - L : (13 - L < 4 ? 4 : (13 - L > 6 ? 6 : 13 - L));
