@@ -24,9 +24,11 @@
 // Two kernels move the values.  col_group_kernel: one thread moves a send
 // buffer into the partner's shared memory with a single bulk copy that
 // completes on the partner's mbarrier, two cluster barriers per round.
-// col_group_l2_kernel (the default): the values go through a scratch block
-// in global memory, resident in L2, one cluster barrier per exchange, and
-// four CTAs exchange once and run both cross stages together (radix 4).
+// col_group_l2_kernel (the faster one; the default for half2 and for wide
+// images of 16384 rows, where col_strip.cu is not faster): the values go
+// through a scratch block in global memory, resident in L2, one cluster
+// barrier per exchange, and four CTAs exchange once and run both cross
+// stages together (radix 4).
 // Only the second has a half2 storage mode (H16): the tile arrives as half2
 // (16-byte TMA box rows) and group 0 widens each value with its row's factor
 // 2^e, as in the single-CTA half2 column pass; at the end every CTA
