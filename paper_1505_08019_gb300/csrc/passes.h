@@ -35,6 +35,9 @@ struct NvtxRange {
 // __restrict__ const pointer, may be fetched before the wait: only a plan's
 // tables are read so, never image data, and chained = false is for callers
 // whose tables the previous kernel has just written.
+// A refused launch (say, a grid beyond the limits) is reported to the caller
+// and taken off the runtime's last error, which the next launch that reads it
+// would otherwise return as its own.
 // cluster > 1: clusters of that many CTAs.
 struct LaunchHow {
     unsigned cluster;
@@ -64,7 +67,10 @@ inline cudaError_t launch_chained(void (*k)(P...), dim3 grid, unsigned block, si
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, k, static_cast<A &&>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, static_cast<A &&>(args)...);
+    if (e != cudaSuccess)
+        cudaGetLastError();
+    return e;
 }
 
 // One int per device (index from device_current(), below 64), computed on
