@@ -304,7 +304,9 @@ FFT2D_API fft2d_status fft2d_exec_host_many_async(int n, const fft2d_plan_t *pla
  * parameter), then one launch per group the column pass -- a handful of
  * launches for any number of images.  In a batch of up to 2^23 pixels one
  * launch per pass serves all lengths (columns of more than 512 rows only
- * while they are few) whose variant was neither tuned nor forced.  Lines of
+ * while they are few) whose variant was not forced
+ * (fft2d_batch_set_variant); a tuned variant is that of its length's own
+ * launch, where the batch takes one.  Lines of
  * 8192 and 16384 points run each image's single-image pass instead, on the
  * group's internal stream.  Every image's result is bit for bit the one
  * fft2d_exec gives.  complex64 plans only.
@@ -463,7 +465,8 @@ FFT2D_API fft2d_status fft2d_exec_noalloc(int rows, int cols, int dir, const voi
  * tiles, persistent TMA-fed with TMA stores, with per-thread stores, or with
  * half of each) and keep the fastest per (pass, axis length) in
  * the process-wide tuning table (and FFT2D_TUNE_CACHE).  Later
- * fft2d_exec_batched calls use the winners.  The buffers are overwritten
+ * fft2d_exec_batched calls use the winners wherever they launch a length by
+ * itself; a batch small enough for one launch over all lengths keeps it.  The buffers are overwritten
  * with intermediate results (the passes run several times).  Synchronous.
  */
 FFT2D_API fft2d_status fft2d_autotune_batched(int n, const fft2d_plan_t *plans,
@@ -474,7 +477,9 @@ FFT2D_API fft2d_status fft2d_autotune_batched(int n, const fft2d_plan_t *plans,
  * name of variant `index` ("" when out of range), the variant the calling
  * thread's current device uses for a pass over lines of 2^L points (-1 on a
  * bad argument or no device), and forcing one (-1: back to the default).  A
- * forced choice goes into the same process-wide table as a tuned winner.  A
+ * forced choice goes into the same process-wide table as a tuned winner (the
+ * next tuning of the length replaces it) and keeps the length out of the
+ * launch that serves all lengths of a small batch.  A
  * variant that cannot serve a group (e.g. the TMA column kernel on an image
  * whose width is not a whole number of tiles) falls back to "plain". */
 FFT2D_API int fft2d_batch_variant_count(int pass);

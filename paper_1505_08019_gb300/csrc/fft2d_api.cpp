@@ -11,8 +11,8 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <set>
 #include <string>
-#include <vector>
 #include <tuple>
 #include <vector>
 
@@ -285,6 +285,8 @@ fft2d_status exec_impl(const fft2d_plan_s *p, const void *in, void *out, int rs,
 // per entry, so that a new process does not have to tune again.
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int>, int> g_tuned;
+// Grouped-launch keys of g_tuned that a caller forced (fft2d_batch_set_variant).
+std::set<std::tuple<int, int, int, int>> g_forced;
 bool g_tune_file_loaded = false;
 
 std::string device_name(int dev)
@@ -569,10 +571,12 @@ fft2d_status batch_groups(int n, const fft2d_plan_t *plans, const void *const *i
 }
 
 // Run the grouped passes of a batch.  A pass's lengths split in two: those of
-// the launch for any length (fft2d::batch_any, unless a variant was tuned or
-// forced for the length), and the rest, one launch per (length, direction)
-// spread over the device's internal lanes.  A pass without a rest needs no
-// lanes and runs on the caller's stream.
+// the launch for any length (fft2d::batch_any, unless a variant was forced for
+// the length), and the rest, one launch per (length, direction) spread over
+// the device's internal lanes.  A pass without a rest needs no lanes and runs
+// on the caller's stream.  A tuned variant says which grouped launch of its
+// length is the fastest, in batches of whatever size the tuner was given; it
+// was not timed against the launch for any length, so it does not replace it.
 fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in,
                          void *const *out, cudaStream_t st)
 {
@@ -598,7 +602,7 @@ fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in
                 if (values[pass][L] == 0)
                     continue;
                 any[pass][L] = fft2d::batch_any(pass == FFT2D_PASS_ROWS, L, values[pass][L], total) &&
-                               !g_tuned.count(std::make_tuple(device, pass + 2, L, 0));
+                               !g_forced.count(std::make_tuple(device, pass + 2, L, 0));
                 (any[pass][L] ? some_any : some_rest)[pass] = true;
             }
     }
@@ -753,7 +757,10 @@ fft2d_status batched_tune(int n, const fft2d_plan_t *plans, const void *const *i
             for (int v = 1; v < (int)tv.size(); v++)
                 if (tv[v] < tv[best])
                     best = v;
-            g_tuned[std::make_tuple(plans[0]->device, kv.first.first + 2, kv.first.second, 0)] = best;
+            const auto key =
+                std::make_tuple(plans[0]->device, kv.first.first + 2, kv.first.second, 0);
+            g_tuned[key] = best;
+            g_forced.erase(key);
         }
         save_tune_file_locked();
     }
@@ -1572,10 +1579,13 @@ fft2d_status fft2d_batch_set_variant(int pass, int L, int variant)
     std::lock_guard<std::mutex> lock(g_tune_mu);
     load_tune_file_locked(dev);
     const auto key = std::make_tuple(dev, pass + 2, L, 0);
-    if (variant < 0)
+    if (variant < 0) {
         g_tuned.erase(key);
-    else
+        g_forced.erase(key);
+    } else {
         g_tuned[key] = variant;
+        g_forced.insert(key);
+    }
     return FFT2D_OK;
 }
 

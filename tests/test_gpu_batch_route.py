@@ -1,0 +1,72 @@
+"""Which launches a batch makes, counted from a captured graph of the call."""
+import ctypes
+
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="no CUDA GPU")]
+
+KERNEL_NODE = 0
+
+
+def launches(call):
+    """Kernel nodes of the graph captured from call(stream)."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph, n = ctypes.c_void_p(), ctypes.c_size_t()
+    assert cu.cuStreamBeginCapture_v2(ctypes.c_void_p(stream.cuda_stream), 1) == 0   # this thread's
+    try:
+        call(stream)
+    finally:
+        ended = cu.cuStreamEndCapture(ctypes.c_void_p(stream.cuda_stream), ctypes.byref(graph))
+    assert ended == 0
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    kinds = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kinds.append(kind.value)
+    cu.cuGraphDestroy(graph)
+    return kinds.count(KERNEL_NODE)
+
+
+def batch(shapes):
+    import paper_1505_08019_gb300 as fft
+    plans = {s: fft.Plan(*s) for s in set(shapes)}
+    xs = [torch.view_as_complex(torch.randn(*s, 2, device="cuda")) for s in shapes]
+    outs = [torch.empty_like(x) for x in xs]
+    handles = [plans[s].handle for s in shapes]
+    fft.fft2d_exec_batched(handles, xs, outs)        # first launches outside the capture
+    return plans, handles, xs, outs
+
+
+def test_tuning_keeps_a_small_batch_in_one_launch_per_pass():
+    import paper_1505_08019_gb300 as fft
+    plans, handles, xs, outs = batch([(64, 128), (128, 64), (64, 64), (128, 128)] * 4)
+
+    def count():
+        return launches(lambda s: fft.fft2d_exec_batched(handles, xs, outs, s))
+
+    want = [o.clone() for o in outs]
+    scratch = [x.clone() for x in xs]
+    try:
+        assert count() == 2
+        fft.fft2d_autotune_batched(handles, scratch, [torch.empty_like(x) for x in xs])
+        assert count() == 2
+        fft.fft2d_exec_batched(handles, xs, outs)
+        assert all(torch.equal(o, w) for o, w in zip(outs, want))
+        # a forced variant is a choice of the length's own launch
+        fft.fft2d_batch_set_variant(fft.FFT2D_PASS_COLS, 6, 1)
+        assert count() == 3
+        fft.fft2d_exec_batched(handles, xs, outs)
+        assert all(torch.equal(o, w) for o, w in zip(outs, want))
+        # and the next tuning replaces it
+        fft.fft2d_autotune_batched(handles, scratch, [torch.empty_like(x) for x in xs])
+        assert count() == 2
+    finally:
+        for length in range(1, 15):
+            for pass_ in (fft.FFT2D_PASS_ROWS, fft.FFT2D_PASS_COLS):
+                fft.fft2d_batch_set_variant(pass_, length, -1)
