@@ -592,7 +592,13 @@ const Variant *select_col_variant(int L, const PassArgs &a)
     const Variant *v = col_variants(L, &n);
     if (!v || n == 0)
         return nullptr;
-    int i = a.variant >= 0 && a.variant < n ? a.variant : col_default_variant(L, a.cols);
+    const bool forced = a.variant >= 0 && a.variant < n;
+    int i = forced ? a.variant : col_default_variant(L, a.cols);
+    // 1024 rows that TMA cannot feed (8-byte aligned buffers, fewer columns
+    // than a tile): tiles of 2^13 values, "narrow" / "plain" in us: 1024x1 6.3 /
+    // 9.4, and from an odd pixel on 1024x8 4.7 / 9.7, 1024x256 5.8 / 7.7
+    if (!forced && L == 10 && !v[i].usable(a))
+        i = ColVariants<10>::index_of("narrow");
     if (!v[i].usable(a))
         i = 0;   // the plain kernel serves every case
     return &v[i];

@@ -1,36 +1,10 @@
 """Which launches a batch makes, counted from a captured graph of the call."""
-import ctypes
-
 import pytest
+
+from _graph import launches
 
 torch = pytest.importorskip("torch")
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="no CUDA GPU")]
-
-KERNEL_NODE = 0
-
-
-def launches(call):
-    """Kernel nodes of the graph captured from call(stream)."""
-    cu = ctypes.CDLL("libcuda.so.1")
-    stream = torch.cuda.Stream()
-    torch.cuda.synchronize()
-    graph, n = ctypes.c_void_p(), ctypes.c_size_t()
-    assert cu.cuStreamBeginCapture_v2(ctypes.c_void_p(stream.cuda_stream), 1) == 0   # this thread's
-    try:
-        call(stream)
-    finally:
-        ended = cu.cuStreamEndCapture(ctypes.c_void_p(stream.cuda_stream), ctypes.byref(graph))
-    assert ended == 0
-    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
-    nodes = (ctypes.c_void_p * n.value)()
-    assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
-    kinds = []
-    for node in nodes:
-        kind = ctypes.c_int()
-        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
-        kinds.append(kind.value)
-    cu.cuGraphDestroy(graph)
-    return kinds.count(KERNEL_NODE)
 
 
 def batch(shapes):
@@ -48,7 +22,7 @@ def test_tuning_keeps_a_small_batch_in_one_launch_per_pass():
     plans, handles, xs, outs = batch([(64, 128), (128, 64), (64, 64), (128, 128)] * 4)
 
     def count():
-        return launches(lambda s: fft.fft2d_exec_batched(handles, xs, outs, s))
+        return len(launches(lambda s: fft.fft2d_exec_batched(handles, xs, outs, s)))
 
     want = [o.clone() for o in outs]
     scratch = [x.clone() for x in xs]
