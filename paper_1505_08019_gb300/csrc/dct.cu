@@ -1627,6 +1627,12 @@ cudaError_t dct_col_strip(bool inverse, int L, const DctIO &d, const float2 *tw,
 // 4096 rows 8.8 against 11.6 (inverse 11.4 / 11.5: stays).  2^13 in the next
 // range: 1024 x 8192 20.7 / 20.8 against 23.4 / 38.5, 2048 x 1024 7.3 / 7.3
 // against 11.8 / 11.5, 4096 x 512 10.0 against 11.8.
+// Wide images of 2048 and 4096 rows that TMA cannot feed (buffers of 8-byte
+// alignment) run tiles of 2^14 values, whose row segments fill whole 32-byte
+// sectors: column pass in us, forward / inverse, against tiles of 2^13: 2048^2
+// 13.1 / 13.4 against 16.2 / 21.9, 2048x8192 45.8 / 46.1 against 45.2 / 53.0,
+// 4096x1024 17.8 / 19.7, 4096^2 57 / 61 (whole transforms 87 / 92 against 97 /
+// 116).
 template <int L>
 using DctTile12 = typename std::conditional<L == 9, LineCfg<9, 3, 0, 32, 5>,
                                             LineCfg<L, (L <= 12 ? 12 - L : 0), 0>>::type;
@@ -1695,6 +1701,9 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
                 const cudaError_t e = idct_col_tma64_launch(d, tw, post, scale, err, 0, s);
                 if (e != cudaErrorNotSupported)
                     return e;
+                if (!col_small_tile((d.cols / 2) << L))
+                    return idct_launch<LineCfg<L, col_kw(L), 0>, false>(d, tw, post, d.cols / 2,
+                                                                        scale, s);
             }
         }
         if constexpr (L == 11) {
@@ -1703,6 +1712,7 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
                     idct_col_tma_launch<LineCfg<L, col_kw(L), 0, 32>>(d, tw, post, scale, err, 0, s);
                 if (e != cudaErrorNotSupported)
                     return e;
+                return idct_launch<LineCfg<L, col_kw(L), 0>, false>(d, tw, post, d.cols / 2, scale, s);
             }
         }
         if constexpr (L >= 6 && L <= 12) {
@@ -1722,6 +1732,7 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
             const cudaError_t e = dct_col_tma64_launch(d, tw, post, scale, err, 0, s);
             if (e != cudaErrorNotSupported)
                 return e;
+            return dct_launch<LineCfg<L, col_kw(L), 0>, false>(d, tw, post, d.cols / 2, scale, s);
         }
     }
     if constexpr (L == 11) {
@@ -1730,6 +1741,7 @@ cudaError_t dct_dispatch(bool row, bool inverse, const DctIO &d, const float2 *t
                 dct_col_tma_launch<LineCfg<L, col_kw(L), 0, 32>>(d, tw, post, scale, err, 0, s);
             if (e != cudaErrorNotSupported)
                 return e;
+            return dct_launch<LineCfg<L, col_kw(L), 0>, false>(d, tw, post, d.cols / 2, scale, s);
         }
     }
     if constexpr (L >= 6 && L <= 12) {

@@ -29,3 +29,28 @@ def test_1024_rows_run_narrow_tiles(cols, odd):
         fft.fft2d_plan_set_variant(p.handle, P, names.index("plain"))
         assert default != geometry(p, plain)
         assert torch.equal(got, narrow) and torch.equal(got, plain)
+
+
+@pytest.mark.parametrize("inverse", [False, True])
+@pytest.mark.parametrize("rows,cols,threads", [(2048, 4, 256), (2048, 1024, 512), (2048, 2048, 1024),
+                                               (4096, 4, 256), (4096, 512, 512), (4096, 1024, 1024),
+                                               (4096, 4096, 1024)])
+def test_dct_tiles_of_long_columns(rows, cols, threads, inverse):
+    """An image of 8-byte alignment: tiles of 2^14 values (16 a thread) where
+    the aligned one is TMA-fed, the smaller tiles of narrow images below that.
+    The result is the aligned one's within the FP32 bound of the other GPU
+    tests."""
+    import paper_1505_08019_gb300 as fft
+    if inverse and (rows, cols) == (4096, 4):
+        threads = 512                  # the inverse has no tiles of 2^12 values here
+    buf = torch.randn(rows * cols + 2, device="cuda")
+    x = buf[2:].view(rows, cols)
+    with fft.Plan(rows, cols, fft.FFT2D_INVERSE if inverse else fft.FFT2D_FORWARD,
+                  fft.FFT2D_R32_DCT2) as p:
+        P = fft.FFT2D_PASS_COLS
+        want, got = torch.empty_like(x), torch.empty_like(buf)[2:].view(rows, cols)
+        fft.fft2d_exec_pass(p.handle, P, x.clone(), want)
+        fft.fft2d_exec_pass(p.handle, P, x, got)
+        (_, block, _), = launches(lambda s: fft.fft2d_exec_pass(p.handle, P, x, got, s))
+        assert block[0] == threads
+        assert float((got - want).norm() / want.norm()) <= 1e-5
