@@ -27,8 +27,8 @@ __device__ __forceinline__ int find_job(const Table &t)
     return lo;
 }
 
-template <bool ROW>
-__global__ void __launch_bounds__(256, 4) batch_any_kernel(const __grid_constant__ BatchTable t)
+template <bool ROW, class Table>
+__global__ void __launch_bounds__(256, 4) batch_any_kernel(const __grid_constant__ Table t)
 {
     const BatchJob &jb = t.job[find_job(t)];
     any_axis<ROW>(jb.L, StoreC64{jb.in, jb.out}, jb.tw, jb.scale, (int)blockIdx.x - jb.first_cta,
@@ -55,15 +55,26 @@ int fill_ctas(Table &t)
     return ctas;
 }
 
-}  // namespace
-
-cudaError_t launch_batch_any(bool row, BatchTable &t, cudaStream_t s)
+template <class Table>
+cudaError_t any_launch(bool row, Table &t, cudaStream_t s)
 {
     const int ctas = fill_ctas(t);
     if (ctas == 0)
         return cudaSuccess;
-    return launch_chained(row ? batch_any_kernel<true> : batch_any_kernel<false>,
+    return launch_chained(row ? batch_any_kernel<true, Table> : batch_any_kernel<false, Table>,
                           dim3((unsigned)ctas), 256, kAnySmem, s, 1, t);
+}
+
+}  // namespace
+
+cudaError_t launch_batch_any(bool row, BatchTable &t, cudaStream_t s)
+{
+    return any_launch(row, t, s);
+}
+
+cudaError_t launch_batch_any(bool row, BatchTableWide &t, cudaStream_t s)
+{
+    return any_launch(row, t, s);
 }
 
 cudaError_t launch_batch_any_h16(bool row, BatchTableH16 &t, int in_axis, cudaStream_t s)

@@ -585,10 +585,13 @@ fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in
         return FFT2D_OK;
     const int device = plans[0]->device;
     long long values[2][15] = {}, total = 0;
+    int jobs[2][15] = {}, any_jobs[2] = {};
     for (int i = 0; i < n; i++) {
         const fft2d_plan_s *p = plans[i];
         if (p->Lr == 0 || p->Lc == 0)
             continue;
+        jobs[0][p->Lc]++;
+        jobs[1][p->Lr]++;
         total += (long long)p->rows * p->cols;
         values[0][p->Lc] += (long long)p->rows * p->cols;
         values[1][p->Lr] += (long long)p->rows * p->cols;
@@ -604,15 +607,16 @@ fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in
                 any[pass][L] = fft2d::batch_any(pass == FFT2D_PASS_ROWS, L, values[pass][L], total) &&
                                !g_forced.count(std::make_tuple(device, pass + 2, L, 0));
                 (any[pass][L] ? some_any : some_rest)[pass] = true;
+                any_jobs[pass] += any[pass][L] ? jobs[pass][L] : 0;
             }
     }
     // every job of the pass's launch for any length, on stream s
-    auto run_any = [&](int pass, cudaStream_t s) {
-        static thread_local fft2d::BatchTable table;
+    auto run_jobs = [&](auto &table, int pass, cudaStream_t s) {
         const bool row = pass == FFT2D_PASS_ROWS;
+        const int most = (int)(sizeof table.job / sizeof table.job[0]);
         table.n = 0;
         for (int i = 0; i <= n; i++) {
-            if ((i == n || table.n == fft2d::kBatchMaxJobs) && table.n > 0) {
+            if ((i == n || table.n == most) && table.n > 0) {
                 const cudaError_t e = fft2d::launch_batch_any(row, table, s);
                 if (e != cudaSuccess)
                     return cuda_fail(e, "batched pass");
@@ -625,6 +629,12 @@ fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in
                 table.job[table.n++] = batch_job(p, row, in[i], out[i]);
         }
         return FFT2D_OK;
+    };
+    auto run_any = [&](int pass, cudaStream_t s) {
+        static thread_local fft2d::BatchTable table;
+        static thread_local fft2d::BatchTableWide wide;
+        return any_jobs[pass] > fft2d::kBatchMaxJobs ? run_jobs(wide, pass, s)
+                                                     : run_jobs(table, pass, s);
     };
     fft2d_status result = FFT2D_OK;
     if (!some_rest[0] && some_any[0])

@@ -208,10 +208,12 @@ struct BatchJob {
     float scale;
     int L;           // log2 of the line length (launch_batch_any)
 };
-struct BatchTable {
+template <int MAX>
+struct BatchTableOf {
     int n;
-    BatchJob job[kBatchMaxJobs];
+    BatchJob job[MAX];
 };
+using BatchTable = BatchTableOf<kBatchMaxJobs>;
 // Job table of the grouped TMA column kernel: a load and a store tensor map
 // per image (a kernel parameter, well inside the 32 KB parameter limit).
 constexpr int kBatchTmaMaxJobs = 64;
@@ -279,6 +281,14 @@ cudaError_t launch_batch_pass(bool row, int L, BatchTable &t, int variant, int *
 // factors.  Lengths 2^1 .. 2^kBatchAnyMaxL.
 constexpr int kBatchAnyMaxL = 12;
 cudaError_t launch_batch_any(bool row, BatchTable &t, cudaStream_t s);
+
+// ... for more than kBatchMaxJobs jobs (24 KB of the 32 KB of parameters).  A
+// second launch starts only when the first has left, and 128 images of 64x512
+// are 1024 CTAs, 1.7 waves: 256 of them took 50.5 us in two launches a pass,
+// 45.4 in one (47.2 with a launch per length); 512 of 128^2 68 and 49, 300 of
+// 32 .. 256 (4.2 M values) 40 and 28.
+using BatchTableWide = BatchTableOf<512>;
+cudaError_t launch_batch_any(bool row, BatchTableWide &t, cudaStream_t s);
 cudaError_t launch_batch_any_h16(bool row, BatchTableH16 &t, int in_axis, cudaStream_t s);
 
 // Whether a group of one axis length (`values` over all its images) joins the
@@ -288,6 +298,11 @@ cudaError_t launch_batch_any_h16(bool row, BatchTableH16 &t, int in_axis, cudaSt
 // 55 M values: 351 against 337 us).  Below: 16 images of 64 .. 128 (0.2 M) 19.9
 // against 33.2 us a call, 10.4 / 13.6 replayed from a graph; 64 images of 128
 // .. 512 (5.8 M) 60 / 84 and 43 / 49; 32 images of 128 .. 1024 (8.5 M) even.
+// Batches of equal images, this launch against a launch per length, at 2^21,
+// 2^22 and 2^23 values: 128^2 16 / 23, 26 / 48, 49 / 90 us; 256^2 14 / 22, 21 /
+// 32, 45 / 58; 512^2 16 / 27, 26 / 41, 52 / 67; 64x512 14 / 21, 22 / 28, 45 / 47;
+// 1024^2, where only the rows join, 23 / 25, 34 / 37, 61 / 60: even at the
+// limit.
 // Rows run the CTAs of their own kernels.  Columns of up to 512 rows join, and
 // longer ones as long as the group fits 128 CTAs of 2^12 values
 // (col_small_tile): beyond that their 32-byte row segments lose to the wider

@@ -44,3 +44,16 @@ def test_tuning_keeps_a_small_batch_in_one_launch_per_pass():
         for length in range(1, 15):
             for pass_ in (fft.FFT2D_PASS_ROWS, fft.FFT2D_PASS_COLS):
                 fft.fft2d_batch_set_variant(pass_, length, -1)
+
+
+@pytest.mark.parametrize("n,want", [(128, 2), (129, 2), (512, 2), (513, 4)])
+def test_a_batch_of_many_images_shares_its_launches(n, want):
+    """Up to 512 images in one launch per pass, each with its own transform's
+    bits, whichever job table holds it."""
+    import paper_1505_08019_gb300 as fft
+    plans, handles, xs, outs = batch([(16, 64), (64, 32), (32, 16)] * (n // 3) + [(8, 128)] * (n % 3))
+    assert len(launches(lambda s: fft.fft2d_exec_batched(handles, xs, outs, s))) == want
+    one = {s: torch.empty(s, dtype=torch.complex64, device="cuda") for s in plans}
+    for x, o in zip(xs, outs):
+        s = tuple(x.shape)
+        assert torch.equal(plans[s](x, one[s]), o)
