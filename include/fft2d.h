@@ -138,10 +138,12 @@ FFT2D_API fft2d_status fft2d_selftest_timeout(fft2d_plan_t plan, void *stream);
  * transform into shared memory): runs the plan's column pass over `in` into
  * `out` (device images of the plan's shape and dtype, row pitch = cols;
  * for FFT2D_R32_DCT2 plans the DCT column pass of the plan's direction,
- * which is TMA-fed for columns of 2048 and 4096 points; plans of 8192 and
- * 16384 rows whose own column pass waits for nothing on the device -- the
- * strip kernel, both dtypes -- run the TMA-fed complex64 cluster pass of that
- * column length instead), except that CTA 0
+ * which is TMA-fed for columns of 2048 and 4096 points).  Two kinds of plans
+ * whose own column pass waits for nothing on the device run another kernel of
+ * their column length instead: 8192 and 16384 rows (the strip kernel, both
+ * dtypes) the TMA-fed complex64 cluster pass, and images narrow enough for
+ * small tiles (2048 rows, both dtypes; DCT of 4096 rows) the TMA-fed kernel
+ * of wider ones.  CTA 0
  * never issues the second TMA load of its
  * first tile.  That CTA's bounded wait gives up after about one second, the
  * kernel records the timeout -- for the cluster kernels of 8192- and

@@ -619,8 +619,6 @@ int col_selftest_variant(int L, const PassArgs &a)
 {
     if (a.variant >= 0)
         return a.variant;
-    if (L == 10)
-        return ColVariants<10>::index_of("narrow");   // refused, as it always was
     if (L == 11)
         return ColVariants<11>::index_of("tma64st");
     if (L == 13)
