@@ -179,7 +179,9 @@ FFT2D_API fft2d_status fft2d_autotune(fft2d_plan_t plan, void *stream);
 /*
  * Write a NUL-terminated description of the kernel variant each pass of the
  * plan uses ("rows:<name>(shape=..,ept=..,tuned|default) cols:...") into
- * buf[0..len).
+ * buf[0..len).  Where fft2d_exec (or fft2d_exec_h16) takes one launch for the
+ * whole image instead of the two passes, " exec:small(ctas=..,ept=..,default)"
+ * follows; the passes named before it are then those of fft2d_exec_pass.
  */
 FFT2D_API fft2d_status fft2d_plan_describe(fft2d_plan_t plan, char *buf, int len);
 

@@ -1186,6 +1186,13 @@ fft2d_status fft2d_plan_describe(fft2d_plan_t p, char *buf, int len)
                       tuned ? "tuned" : "default");
         out += tmp;
     }
+    // the whole transform of a small image: one launch instead of the passes
+    const bool half2 = p->dtype == FFT2D_C32H;
+    const int ctas = half2 || (p->row_variant < 0 && p->col_variant < 0)
+                         ? fft2d::small_image_ctas(half2, p->Lr, p->Lc)
+                         : 0;
+    if (ctas > 0)
+        out += " exec:small(ctas=" + std::to_string(ctas) + ",ept=16,default)";
     std::snprintf(buf, (size_t)len, "%s", out.c_str());
     return FFT2D_OK;
 }

@@ -187,6 +187,8 @@ struct SmallArgs {
     float scale;
 };
 bool small_image(int Lr, int Lc);
+// The CTAs of that launch on the current device, 0 where it is not taken.
+int small_image_ctas(bool half2, int Lr, int Lc);
 cudaError_t launch_small(const SmallArgs &a, const float2 *in, float2 *out, cudaStream_t s);
 cudaError_t launch_small_h16(const SmallArgs &a, const __half2 *in, const int *in_exp, int in_axis,
                              __half2 *out, int *row_exp, int *out_exp, cudaStream_t s);

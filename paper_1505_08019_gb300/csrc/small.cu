@@ -49,41 +49,51 @@ __global__ void __launch_bounds__(256, 4) small_kernel(const RIO rio, const CIO 
     any_axis<false>(Lr, cio, tw_cols, scale, cta, cols, cols);
 }
 
+int small_ctas(int Lr, int Lc) { return Lr + Lc > kAnyL ? 1 << (Lr + Lc - kAnyL) : 1; }
+
+// Whether the device takes the kernel in clusters of `ctas`: above 8 they are
+// opt-in, and a device may refuse them.
+template <class RIO, class CIO>
+bool small_cluster_ok(int ctas)
+{
+    if (ctas <= 8)
+        return true;
+    auto k = small_kernel<RIO, CIO>;
+    static DeviceCache ok;   // 1: usable, 2: not
+    const int d = device_current();
+    if (!ok.get(d)) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        int n = 0;
+        if (e == cudaSuccess) {
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = kSmallMaxCtas;
+            at[0].val.clusterDim.y = 1;
+            at[0].val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(kSmallMaxCtas);
+            cfg.blockDim = dim3(256);
+            cfg.dynamicSmemBytes = kAnySmem;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
+        }
+        if (e != cudaSuccess)
+            cudaGetLastError();
+        ok.set(d, e == cudaSuccess && n > 0 ? 1 : 2);
+    }
+    return ok.get(d) == 1;
+}
+
 template <class RIO, class CIO>
 cudaError_t small_launch(const RIO &rio, const CIO &cio, const SmallArgs &a, cudaStream_t s)
 {
-    auto k = small_kernel<RIO, CIO>;
-    const int ctas = a.Lr + a.Lc > kAnyL ? 1 << (a.Lr + a.Lc - kAnyL) : 1;
-    if (ctas > 8) {
-        // clusters above 8 CTAs are opt-in, and a device may refuse them
-        static DeviceCache ok;   // 1: usable, 2: not
-        const int d = device_current();
-        if (!ok.get(d)) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-            int n = 0;
-            if (e == cudaSuccess) {
-                cudaLaunchAttribute at[1];
-                at[0].id = cudaLaunchAttributeClusterDimension;
-                at[0].val.clusterDim.x = kSmallMaxCtas;
-                at[0].val.clusterDim.y = 1;
-                at[0].val.clusterDim.z = 1;
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3(kSmallMaxCtas);
-                cfg.blockDim = dim3(256);
-                cfg.dynamicSmemBytes = kAnySmem;
-                cfg.attrs = at;
-                cfg.numAttrs = 1;
-                e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
-            }
-            if (e != cudaSuccess)
-                cudaGetLastError();
-            ok.set(d, e == cudaSuccess && n > 0 ? 1 : 2);
-        }
-        if (ok.get(d) != 1)
-            return cudaErrorNotSupported;
-    }
-    return launch_chained(k, dim3(ctas), 256, kAnySmem, s, LaunchHow((unsigned)ctas), rio, cio,
-                          a.tw_rows, a.tw_cols, 1 << a.Lr, 1 << a.Lc, a.Lr, a.Lc, a.scale);
+    const int ctas = small_ctas(a.Lr, a.Lc);
+    if (!small_cluster_ok<RIO, CIO>(ctas))
+        return cudaErrorNotSupported;
+    return launch_chained(small_kernel<RIO, CIO>, dim3(ctas), 256, kAnySmem, s,
+                          LaunchHow((unsigned)ctas), rio, cio, a.tw_rows, a.tw_cols, 1 << a.Lr,
+                          1 << a.Lc, a.Lr, a.Lc, a.scale);
 }
 
 }  // namespace
@@ -92,6 +102,16 @@ cudaError_t small_launch(const RIO &rio, const CIO &cio, const SmallArgs &a, cud
 bool small_image(int Lr, int Lc)
 {
     return Lr >= 1 && Lc >= 1 && Lr <= kAnyL && Lc <= kAnyL && Lr + Lc <= kAnyL + 4;
+}
+
+int small_image_ctas(bool half2, int Lr, int Lc)
+{
+    if (!small_image(Lr, Lc))
+        return 0;
+    const int ctas = small_ctas(Lr, Lc);
+    const bool ok = half2 ? small_cluster_ok<StoreH16T<0>, StoreH16Shared<0>>(ctas)
+                          : small_cluster_ok<StoreC64, StoreC64Shared>(ctas);
+    return ok ? ctas : 0;
 }
 
 cudaError_t launch_small(const SmallArgs &a, const float2 *in, float2 *out, cudaStream_t s)
