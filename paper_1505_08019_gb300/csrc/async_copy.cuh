@@ -24,9 +24,10 @@ constexpr unsigned kPollSuspendNs = 1000;
 constexpr int kDevErrTmaTimeout = 1;
 
 // Wait until every kernel this one was launched behind (launch_chained) has
-// finished and its writes are visible.  A kernel calls it before its first
-// access to global memory, with all its threads; launched any other way it
-// returns at once.
+// finished and its writes are visible.  Every thread calls it before the
+// kernel's first access to image data, exponents or scratch; before it a
+// kernel reads at most a plan's tables, its parameters and shared memory.
+// Launched any other way it returns at once.
 __device__ __forceinline__ void pdl_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -10,6 +10,7 @@
 // so a batched image is bit-for-bit the image transformed alone.
 #include <type_traits>
 
+#include "batch_job.cuh"
 #include "line_fft.cuh"
 #include "passes.h"
 
@@ -21,21 +22,6 @@ namespace {
 // GPU, where the single-image pass's smaller CTAs lose (64 images of 128 ..
 // 2048: 280 against 275 us).
 constexpr int batch_row_kb(int L) { return L <= 12 ? 12 - L : 0; }
-
-template <class Table>
-__device__ __forceinline__ int find_job(const Table &t)
-{
-    int lo = 0, hi = t.n - 1;
-    const int b = (int)blockIdx.x;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (t.job[mid].first_cta <= b)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
 
 template <class C>
 __global__ void __launch_bounds__(C::T, C::MINB) row_batch_kernel(const __grid_constant__ BatchTable t)

@@ -5,27 +5,12 @@
 // launches and events on the host and by the gaps between small kernels on
 // the device, not by its traffic.
 #include "any_axis.cuh"
+#include "batch_job.cuh"
 #include "passes.h"
 
 namespace fft2d {
 
 namespace {
-
-// Index of the job that owns this CTA.
-template <class Table>
-__device__ __forceinline__ int find_job(const Table &t)
-{
-    int lo = 0, hi = t.n - 1;
-    const int b = (int)blockIdx.x;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (t.job[mid].first_cta <= b)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
 
 template <bool ROW, class Table>
 __global__ void __launch_bounds__(256, 4) batch_any_kernel(const __grid_constant__ Table t)

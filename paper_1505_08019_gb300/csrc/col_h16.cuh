@@ -2,9 +2,10 @@
 // power-of-two exponent per line, FP32 arithmetic).
 //
 // The arithmetic is the FP32 column engine's (a tile of W = 4 or 8 whole
-// columns of 2^L rows in two groups of radix-2 DIT stages, Section 2 eqs. 2-3 / Section 3.1 eq. 4, the scramble of Section 3.2 fused
-// into the first read), so the results are those of the complex64 column
-// pass on the dequantised input, rounded once to half precision at the end.
+// columns of 2^L rows in two groups of radix-2 DIT stages, Section 2 eqs. 2-3 /
+// Section 3.1 eq. 4, the scramble of Section 3.2 fused into the first read),
+// so the results are those of the complex64 column pass on the dequantised
+// input, rounded once to half precision at the end.
 // Only the storage differs:
 //
 //  * The tile arrives as half2 (4 bytes a pixel): its first half (the early

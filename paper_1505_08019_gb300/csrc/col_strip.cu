@@ -138,213 +138,220 @@ __global__ void __launch_bounds__(256, 4) col_strip_kernel(const StripArgs g)
     float2 a[16];
     float2 *slot = (phase ? g.scratch[1] : g.scratch[0]) + rel * S::SLOT;
     if (phase == 0) {
-            if (tid < S::NA - 1)
-                tw1[tid] = __ldg(g.tw + tid);   // read after the exchange barrier
-            constexpr int W = S::W1;         // 16: half-warps run over columns
-            const int w = tid % W, u = tid / W;
-            const int pi = idx / (kStripCols / W);
-            const int wb = idx % (kStripCols / W) * W + w;    // column of the strip
-            const int col = strip * kStripCols + wb;
-            const bool live = col < g.cols;
-            const int c0 = pi, c1 = pi == 0 ? NB / 2 : NB - pi;  // the two residues
-            const float2 *src = g.in + col;
-            if constexpr (MODE == kStripIdct) {
-                // units (c0, hib) and (c1, 15 - hib), 3 stages; position
-                // index r holds row c + NB i, i = rev3(r) 16 | hib
-                const float2 z = make_float2(0.f, 0.f);
+        if (tid < S::NA - 1)
+            tw1[tid] = __ldg(g.tw + tid);   // read after the exchange barrier
+        constexpr int W = S::W1;         // 16: half-warps run over columns
+        const int w = tid % W, u = tid / W;
+        const int pi = idx / (kStripCols / W);
+        const int wb = idx % (kStripCols / W) * W + w;    // column of the strip
+        const int col = strip * kStripCols + wb;
+        const bool live = col < g.cols;
+        const int c0 = pi, c1 = pi == 0 ? NB / 2 : NB - pi;  // the two residues
+        const float2 *src = g.in + col;
+        if constexpr (MODE == kStripIdct) {
+            // units (c0, hib) and (c1, 15 - hib), 3 stages; position
+            // index r holds row c + NB i, i = rev3(r) 16 | hib
+            const float2 z = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < 8; r++) {
+                const int i0 = brev_c(r, 3) * 16 + u, i1 = brev_c(r, 3) * 16 + 15 - u;
+                a[r] = live ? ld_stream(src + (long long)(c0 + NB * i0) * g.ld) : z;
+                a[8 + r] = live ? ld_stream(src + (long long)(c1 + NB * i1) * g.ld) : z;
+            }
+            if (pi != 0) {
 #pragma unroll
                 for (int r = 0; r < 8; r++) {
-                    const int i0 = brev_c(r, 3) * 16 + u, i1 = brev_c(r, 3) * 16 + 15 - u;
-                    a[r] = live ? ld_stream(src + (long long)(c0 + NB * i0) * g.ld) : z;
-                    a[8 + r] = live ? ld_stream(src + (long long)(c1 + NB * i1) * g.ld) : z;
+                    const int k = c0 + NB * (brev_c(r, 3) * 16 + u);
+                    const float2 x0 = a[r], x1 = a[15 - r];       // k and N - k
+                    if (r % 2 == 0)                                // k < N/2
+                        idct_pre(x0, x1, __ldg(g.post + k), a[r], a[15 - r]);
+                    else
+                        idct_pre(x1, x0, __ldg(g.post + (N - k)), a[15 - r], a[r]);
                 }
-                if (pi != 0) {
-#pragma unroll
-                    for (int r = 0; r < 8; r++) {
-                        const int k = c0 + NB * (brev_c(r, 3) * 16 + u);
-                        const float2 x0 = a[r], x1 = a[15 - r];       // k and N - k
-                        if (r % 2 == 0)                                // k < N/2
-                            idct_pre(x0, x1, __ldg(g.post + k), a[r], a[15 - r]);
-                        else
-                            idct_pre(x1, x0, __ldg(g.post + (N - k)), a[15 - r], a[r]);
-                    }
-                } else {
-                    // residues 0 and NB/2 are their own mirrors, in other
-                    // threads: partners through shared memory
-#pragma unroll
-                    for (int j = 0; j < 16; j++) {
-                        const int i = brev_c(j % 8, 3) * 16 + (j < 8 ? u : 15 - u);
-                        sm[(j / 8 << LA | i) * W + w] = a[j];
-                    }
-                    __syncthreads();
-#pragma unroll
-                    for (int j = 0; j < 16; j++) {
-                        const int i = brev_c(j % 8, 3) * 16 + (j < 8 ? u : 15 - u);
-                        const int im = j < 8 ? (S::NA - i) & (S::NA - 1) : S::NA - 1 - i;
-                        const int k = (j < 8 ? 0 : NB / 2) + NB * i;
-                        if (k == 0)
-                            continue;                                  // X[N] = 0
-                        const float2 o = sm[(j / 8 << LA | im) * W + w];
-                        float2 yk, yp;
-                        if (k <= N / 2) {
-                            idct_pre(a[j], o, __ldg(g.post + k), yk, yp);
-                            a[j] = yk;
-                        } else {
-                            idct_pre(o, a[j], __ldg(g.post + (N - k)), yk, yp);
-                            a[j] = yp;
-                        }
-                    }
-                    __syncthreads();
-                }
-#pragma unroll
-                for (int v = 0; v < 2; v++) {
-                    unit_stages<3, true>(a, 8 * v, p, [&](int t, int m) { return __ldg(g.tw + (1 << t) - 1 + m); });
-                    const int hi = brev_rt(v ? 15 - u : u, 4);
-#pragma unroll
-                    for (int r = 0; r < 8; r++)
-                        sm[((v << LA) | r | (hi << 3)) * W + w] = a[8 * v + r];
-                }
-                __syncthreads();
-                const int set = u >> 3, lo = u & 7;
-#pragma unroll
-                for (int r = 0; r < 16; r++)
-                    a[r] = sm[((set << LA) | lo | (r << 3)) * W + w];
-                unit_stages<4, false>(a, 0, p, [&](int t, int m) { return tw1[(8 << t) - 1 + lo + 8 * m]; });
-                const int b = brev_rt(set ? c1 : c0, LB);
-                float2 *dst = slot + ((b << LA) | lo) * kStripCols + wb;
-#pragma unroll
-                for (int r = 0; r < 16; r++)
-                    dst[(r << 3) * kStripCols] = a[r];
             } else {
-                // unit (set, hib), 4 stages; index r holds element
-                // n = c + NB i, i = rev4(r) 8 | hib
-                const int set = u >> 3, hib = u & 7;
-                const int c = set ? c1 : c0;
-#pragma unroll
-                for (int r = 0; r < 16; r++) {
-                    const int n = c + NB * (brev_c(r, 4) * 8 + hib);
-                    const int row = MODE == kStripDct ? dct_row<N>(n, r % 2 == 0) : n;
-                    a[r] = live ? ld_stream(src + (long long)row * g.ld) : make_float2(0.f, 0.f);
-                }
-                unit_stages<4, true>(a, 0, p, [&](int t, int m) { return __ldg(g.tw + (1 << t) - 1 + m); });
-                const int hi = brev_rt(hib, 3);
-#pragma unroll
-                for (int r = 0; r < 16; r++)
-                    sm[((set << LA) | r | (hi << 4)) * W + w] = a[r];
-                __syncthreads();
-#pragma unroll
-                for (int v = 0; v < 2; v++) {
-#pragma unroll
-                    for (int r = 0; r < 8; r++)
-                        a[8 * v + r] = sm[((v << LA) | u | (r << 4)) * W + w];
-                    unit_stages<3, false>(a, 8 * v, p, [&](int t, int m) { return tw1[(16 << t) - 1 + u + 16 * m]; });
-                    const int b = brev_rt(v ? c1 : c0, LB);
-                    float2 *dst = slot + ((b << LA) | u) * kStripCols + wb;
-#pragma unroll
-                    for (int r = 0; r < 8; r++)
-                        dst[(r << 4) * kStripCols] = a[8 * v + r];
-                }
-            }
-        } else {
-            constexpr int W = S::W2;         // 16, or a whole warp of columns
-            const int w = tid % W, u = tid / W;
-            const int li = idx / (kStripCols / W);
-            const int wb = idx % (kStripCols / W) * W + w;
-            const int col = strip * kStripCols + wb;
-            const bool live = col < g.cols;
-            const int lo0 = li, lo1 = li == 0 ? S::NA / 2 : S::NA - li;
-            // value index j of this thread: unit v = j / 8 (7 + 7: one unit
-            // of 16), scratch row lo + 2^LA b
-#pragma unroll
-            for (int j = 0; j < 16; j++) {
-                const int set = LB == 7 ? u >> 3 : j / 8;
-                const int b = LB == 7 ? j | (u & 7) << 4 : j % 8 | u << 3;
-                a[j] = ld_l2(slot + ((b << LA) | (set ? lo1 : lo0)) * kStripCols + wb);
-            }
-            if (tid < 2 * (NB - 1)) {
-                const int set = tid / (NB - 1), e = tid % (NB - 1) + 1;
-                const int t = 31 - __clz(e), m = e - (1 << t);
-                tw2[set * NB + e - 1] =
-                    __ldg(g.tw + (S::NA << t) - 1 + (set ? lo1 : lo0) + S::NA * m);
-            }
-            __syncthreads();
-            if constexpr (LB == 7) {
-                const int set = u >> 3, rhi = u & 7;
-                unit_stages<4, false>(a, 0, p, [&](int t, int m) { return tw2[set * NB + (1 << t) - 1 + m]; });
-#pragma unroll
-                for (int r = 0; r < 16; r++)
-                    sm[((set << LB) | r | (rhi << 4)) * W + w] = a[r];
-            } else {
-#pragma unroll
-                for (int v = 0; v < 2; v++) {
-                    unit_stages<3, false>(a, 8 * v, p, [&](int t, int m) { return tw2[v * NB + (1 << t) - 1 + m]; });
-#pragma unroll
-                    for (int r = 0; r < 8; r++)
-                        sm[((v << LB) | r | (u << 3)) * W + w] = a[8 * v + r];
-                }
-            }
-            __syncthreads();
-            // last three stages: units (lo0, rl) and (lo1, mirrored rl)
-            constexpr int GL = LB - 3, RL = 1 << GL;
-#pragma unroll
-            for (int v = 0; v < 2; v++) {
-                const int rl = v ? RL - 1 - u : u;
-#pragma unroll
-                for (int r = 0; r < 8; r++)
-                    a[8 * v + r] = sm[((v << LB) | rl | (r << GL)) * W + w];
-                unit_stages<3, false>(a, 8 * v, p, [&](int t, int m) { return tw2[v * NB + (RL << t) - 1 + rl + RL * m]; });
-            }
-            float2 *dst = g.out + col;
-            if constexpr (MODE == kStripDct) {
-                // output K = lo + 2^LA b, partner N - K: index 15 - j of the
-                // same thread, or (lo 0 and 2^LA / 2) through shared memory
-                if (li != 0) {
-#pragma unroll
-                    for (int r = 0; r < 8; r++) {
-                        const int K = lo0 + S::NA * (u | r << GL);
-                        const float2 x0 = a[r], x1 = a[15 - r];
-                        if (r < 4)                                   // K < N/2
-                            dct_pair(x0, x1, __ldg(g.post + K), g.scale, a[r], a[15 - r]);
-                        else
-                            dct_pair(x1, x0, __ldg(g.post + (N - K)), g.scale, a[15 - r], a[r]);
-                    }
-                } else {
-                    __syncthreads();
-#pragma unroll
-                    for (int j = 0; j < 16; j++) {
-                        const int v = j / 8, rl = v ? RL - 1 - u : u;
-                        sm[((v << LB) | rl | ((j % 8) << GL)) * W + w] = a[j];
-                    }
-                    __syncthreads();
-#pragma unroll
-                    for (int j = 0; j < 16; j++) {
-                        const int v = j / 8, rl = v ? RL - 1 - u : u;
-                        const int b = rl | (j % 8) << GL;
-                        const int K = (v ? lo1 : 0) + S::NA * b;
-                        const int bm = v ? NB - 1 - b : (NB - b) & (NB - 1);
-                        const float2 o = sm[((v << LB) | bm) * W + w];
-                        float2 xk, xp;
-                        if (K <= N / 2) {
-                            dct_pair(a[j], o, __ldg(g.post + K), g.scale, xk, xp);
-                            a[j] = xk;
-                        } else {
-                            dct_pair(o, a[j], __ldg(g.post + (N - K)), g.scale, xk, xp);
-                            a[j] = xp;
-                        }
-                    }
-                }
-            }
-            if (live) {
+                // residues 0 and NB/2 are their own mirrors, in other
+                // threads: partners through shared memory
 #pragma unroll
                 for (int j = 0; j < 16; j++) {
-                    const int v = j / 8, r = j % 8, rl = v ? RL - 1 - u : u;
-                    const int n = (v ? lo1 : lo0) + S::NA * (rl | r << GL);
-                    const int row = MODE == kStripIdct ? dct_row<N>(n, r < 4) : n;
-                    const float f = MODE == kStripDct ? 1.f : g.scale;
-                    st_stream(dst + (long long)row * g.ld, make_float2(a[j].x * f, a[j].y * f));
+                    const int i = brev_c(j % 8, 3) * 16 + (j < 8 ? u : 15 - u);
+                    sm[(j / 8 << LA | i) * W + w] = a[j];
+                }
+                __syncthreads();
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    const int i = brev_c(j % 8, 3) * 16 + (j < 8 ? u : 15 - u);
+                    const int im = j < 8 ? (S::NA - i) & (S::NA - 1) : S::NA - 1 - i;
+                    const int k = (j < 8 ? 0 : NB / 2) + NB * i;
+                    if (k == 0)
+                        continue;                                  // X[N] = 0
+                    const float2 o = sm[(j / 8 << LA | im) * W + w];
+                    float2 yk, yp;
+                    if (k <= N / 2) {
+                        idct_pre(a[j], o, __ldg(g.post + k), yk, yp);
+                        a[j] = yk;
+                    } else {
+                        idct_pre(o, a[j], __ldg(g.post + (N - k)), yk, yp);
+                        a[j] = yp;
+                    }
+                }
+                __syncthreads();
+            }
+#pragma unroll
+            for (int v = 0; v < 2; v++) {
+                unit_stages<3, true>(a, 8 * v, p,
+                                     [&](int t, int m) { return __ldg(g.tw + (1 << t) - 1 + m); });
+                const int hi = brev_rt(v ? 15 - u : u, 4);
+#pragma unroll
+                for (int r = 0; r < 8; r++)
+                    sm[((v << LA) | r | (hi << 3)) * W + w] = a[8 * v + r];
+            }
+            __syncthreads();
+            const int set = u >> 3, lo = u & 7;
+#pragma unroll
+            for (int r = 0; r < 16; r++)
+                a[r] = sm[((set << LA) | lo | (r << 3)) * W + w];
+            unit_stages<4, false>(a, 0, p,
+                                  [&](int t, int m) { return tw1[(8 << t) - 1 + lo + 8 * m]; });
+            const int b = brev_rt(set ? c1 : c0, LB);
+            float2 *dst = slot + ((b << LA) | lo) * kStripCols + wb;
+#pragma unroll
+            for (int r = 0; r < 16; r++)
+                dst[(r << 3) * kStripCols] = a[r];
+        } else {
+            // unit (set, hib), 4 stages; index r holds element
+            // n = c + NB i, i = rev4(r) 8 | hib
+            const int set = u >> 3, hib = u & 7;
+            const int c = set ? c1 : c0;
+#pragma unroll
+            for (int r = 0; r < 16; r++) {
+                const int n = c + NB * (brev_c(r, 4) * 8 + hib);
+                const int row = MODE == kStripDct ? dct_row<N>(n, r % 2 == 0) : n;
+                a[r] = live ? ld_stream(src + (long long)row * g.ld) : make_float2(0.f, 0.f);
+            }
+            unit_stages<4, true>(a, 0, p,
+                                 [&](int t, int m) { return __ldg(g.tw + (1 << t) - 1 + m); });
+            const int hi = brev_rt(hib, 3);
+#pragma unroll
+            for (int r = 0; r < 16; r++)
+                sm[((set << LA) | r | (hi << 4)) * W + w] = a[r];
+            __syncthreads();
+#pragma unroll
+            for (int v = 0; v < 2; v++) {
+#pragma unroll
+                for (int r = 0; r < 8; r++)
+                    a[8 * v + r] = sm[((v << LA) | u | (r << 4)) * W + w];
+                unit_stages<3, false>(a, 8 * v, p,
+                                      [&](int t, int m) { return tw1[(16 << t) - 1 + u + 16 * m]; });
+                const int b = brev_rt(v ? c1 : c0, LB);
+                float2 *dst = slot + ((b << LA) | u) * kStripCols + wb;
+#pragma unroll
+                for (int r = 0; r < 8; r++)
+                    dst[(r << 4) * kStripCols] = a[8 * v + r];
+            }
+        }
+    } else {
+        constexpr int W = S::W2;         // 16, or a whole warp of columns
+        const int w = tid % W, u = tid / W;
+        const int li = idx / (kStripCols / W);
+        const int wb = idx % (kStripCols / W) * W + w;
+        const int col = strip * kStripCols + wb;
+        const bool live = col < g.cols;
+        const int lo0 = li, lo1 = li == 0 ? S::NA / 2 : S::NA - li;
+        // value index j of this thread: unit v = j / 8 (7 + 7: one unit
+        // of 16), scratch row lo + 2^LA b
+#pragma unroll
+        for (int j = 0; j < 16; j++) {
+            const int set = LB == 7 ? u >> 3 : j / 8;
+            const int b = LB == 7 ? j | (u & 7) << 4 : j % 8 | u << 3;
+            a[j] = ld_l2(slot + ((b << LA) | (set ? lo1 : lo0)) * kStripCols + wb);
+        }
+        if (tid < 2 * (NB - 1)) {
+            const int set = tid / (NB - 1), e = tid % (NB - 1) + 1;
+            const int t = 31 - __clz(e), m = e - (1 << t);
+            tw2[set * NB + e - 1] =
+                __ldg(g.tw + (S::NA << t) - 1 + (set ? lo1 : lo0) + S::NA * m);
+        }
+        __syncthreads();
+        if constexpr (LB == 7) {
+            const int set = u >> 3, rhi = u & 7;
+            unit_stages<4, false>(a, 0, p,
+                                  [&](int t, int m) { return tw2[set * NB + (1 << t) - 1 + m]; });
+#pragma unroll
+            for (int r = 0; r < 16; r++)
+                sm[((set << LB) | r | (rhi << 4)) * W + w] = a[r];
+        } else {
+#pragma unroll
+            for (int v = 0; v < 2; v++) {
+                unit_stages<3, false>(a, 8 * v, p,
+                                      [&](int t, int m) { return tw2[v * NB + (1 << t) - 1 + m]; });
+#pragma unroll
+                for (int r = 0; r < 8; r++)
+                    sm[((v << LB) | r | (u << 3)) * W + w] = a[8 * v + r];
+            }
+        }
+        __syncthreads();
+        // last three stages: units (lo0, rl) and (lo1, mirrored rl)
+        constexpr int GL = LB - 3, RL = 1 << GL;
+#pragma unroll
+        for (int v = 0; v < 2; v++) {
+            const int rl = v ? RL - 1 - u : u;
+#pragma unroll
+            for (int r = 0; r < 8; r++)
+                a[8 * v + r] = sm[((v << LB) | rl | (r << GL)) * W + w];
+            unit_stages<3, false>(a, 8 * v, p,
+                                  [&](int t, int m) { return tw2[v * NB + (RL << t) - 1 + rl + RL * m]; });
+        }
+        float2 *dst = g.out + col;
+        if constexpr (MODE == kStripDct) {
+            // output K = lo + 2^LA b, partner N - K: index 15 - j of the
+            // same thread, or (lo 0 and 2^LA / 2) through shared memory
+            if (li != 0) {
+#pragma unroll
+                for (int r = 0; r < 8; r++) {
+                    const int K = lo0 + S::NA * (u | r << GL);
+                    const float2 x0 = a[r], x1 = a[15 - r];
+                    if (r < 4)                                   // K < N/2
+                        dct_pair(x0, x1, __ldg(g.post + K), g.scale, a[r], a[15 - r]);
+                    else
+                        dct_pair(x1, x0, __ldg(g.post + (N - K)), g.scale, a[15 - r], a[r]);
+                }
+            } else {
+                __syncthreads();
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    const int v = j / 8, rl = v ? RL - 1 - u : u;
+                    sm[((v << LB) | rl | ((j % 8) << GL)) * W + w] = a[j];
+                }
+                __syncthreads();
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    const int v = j / 8, rl = v ? RL - 1 - u : u;
+                    const int b = rl | (j % 8) << GL;
+                    const int K = (v ? lo1 : 0) + S::NA * b;
+                    const int bm = v ? NB - 1 - b : (NB - b) & (NB - 1);
+                    const float2 o = sm[((v << LB) | bm) * W + w];
+                    float2 xk, xp;
+                    if (K <= N / 2) {
+                        dct_pair(a[j], o, __ldg(g.post + K), g.scale, xk, xp);
+                        a[j] = xk;
+                    } else {
+                        dct_pair(o, a[j], __ldg(g.post + (N - K)), g.scale, xk, xp);
+                        a[j] = xp;
+                    }
                 }
             }
         }
+        if (live) {
+#pragma unroll
+            for (int j = 0; j < 16; j++) {
+                const int v = j / 8, r = j % 8, rl = v ? RL - 1 - u : u;
+                const int n = (v ? lo1 : lo0) + S::NA * (rl | r << GL);
+                const int row = MODE == kStripIdct ? dct_row<N>(n, r < 4) : n;
+                const float f = MODE == kStripDct ? 1.f : g.scale;
+                st_stream(dst + (long long)row * g.ld, make_float2(a[j].x * f, a[j].y * f));
+            }
+        }
+    }
 }
 
 template <int MODE, int LA, int LB>

@@ -595,7 +595,8 @@ cudaError_t row_dct_launch(const DctIO &d, const float2 *tw, const float2 *post,
             return e;
     }
     const unsigned grid = (unsigned)((nlines + C::LB - 1) / C::LB);
-    return launch_chained(k, (unsigned)grid, C::T, bytes, s, 1, d, tw, post, dct_rot_table(), nlines, scale);
+    return launch_chained(k, (unsigned)grid, C::T, bytes, s, 1, d, tw, post, dct_rot_table(),
+                          nlines, scale);
 }
 
 // ---------------------------------------------------------------------------
@@ -823,7 +824,8 @@ cudaError_t dct_col_tma_launch(const DctIO &d, const float2 *tw, const float2 *p
     int grid = device_sm_count();
     if (grid > ntiles)
         grid = ntiles;
-    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, me, mo, omap, out, cc, ntiles, tw, post, dct_rot_table(), scale, err, withhold);
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, me, mo, omap, out, cc, ntiles, tw,
+                          post, dct_rot_table(), scale, err, withhold);
 }
 
 // ---------------------------------------------------------------------------
@@ -1054,7 +1056,8 @@ cudaError_t dct_col_tma64_launch(const DctIO &d, const float2 *tw, const float2 
     int grid = device_sm_count();
     if (grid > ntiles)
         grid = ntiles;
-    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, me, mo, omap, ntiles, tw, post, scale, err, withhold);
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, me, mo, omap, ntiles, tw, post,
+                          scale, err, withhold);
 }
 
 // ---------------------------------------------------------------------------
@@ -1243,7 +1246,8 @@ cudaError_t idct_col_tma64_launch(const DctIO &d, const float2 *tw, const float2
     int grid = device_sm_count();
     if (grid > ntiles)
         grid = ntiles;
-    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, oe, oo, ntiles, tw, post, scale, err, withhold);
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, oe, oo, ntiles, tw, post, scale,
+                          err, withhold);
 }
 
 template <class C, bool ROW>
@@ -1422,7 +1426,8 @@ cudaError_t row_idct_launch(const DctIO &d, const float2 *tw, const float2 *post
             return e;
     }
     const unsigned grid = (unsigned)((nlines + C::LB - 1) / C::LB);
-    return launch_chained(k, (unsigned)grid, C::T, bytes, s, 1, d, tw, post, dct_rot_table(), nlines, scale);
+    return launch_chained(k, (unsigned)grid, C::T, bytes, s, 1, d, tw, post, dct_rot_table(),
+                          nlines, scale);
 }
 
 // Inverse column pass, persistent and TMA-fed like the complex column pass
@@ -1605,7 +1610,8 @@ cudaError_t idct_col_tma_launch(const DctIO &d, const float2 *tw, const float2 *
     int grid = device_sm_count();
     if (grid > ntiles)
         grid = ntiles;
-    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, oe, out, cc, ntiles, tw, post, dct_rot_table(), scale, err, withhold);
+    return launch_chained(k, (unsigned)grid, C::T, SMEM, s, 1, map, oe, out, cc, ntiles, tw, post,
+                          dct_rot_table(), scale, err, withhold);
 }
 
 cudaError_t dct_col_strip(bool inverse, int L, const DctIO &d, const float2 *tw, const float2 *post,
