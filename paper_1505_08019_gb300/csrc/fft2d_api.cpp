@@ -585,13 +585,14 @@ fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in
         return FFT2D_OK;
     const int device = plans[0]->device;
     long long values[2][15] = {}, total = 0;
-    int jobs[2][15] = {}, any_jobs[2] = {};
+    int jobs[2][15][2] = {};   // by direction
+    int any_jobs[2] = {}, rest_launches[2] = {};
     for (int i = 0; i < n; i++) {
         const fft2d_plan_s *p = plans[i];
         if (p->Lr == 0 || p->Lc == 0)
             continue;
-        jobs[0][p->Lc]++;
-        jobs[1][p->Lr]++;
+        jobs[0][p->Lc][p->dir > 0]++;
+        jobs[1][p->Lr][p->dir > 0]++;
         total += (long long)p->rows * p->cols;
         values[0][p->Lc] += (long long)p->rows * p->cols;
         values[1][p->Lr] += (long long)p->rows * p->cols;
@@ -607,7 +608,13 @@ fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in
                 any[pass][L] = fft2d::batch_any(pass == FFT2D_PASS_ROWS, L, values[pass][L], total) &&
                                !g_forced.count(std::make_tuple(device, pass + 2, L, 0));
                 (any[pass][L] ? some_any : some_rest)[pass] = true;
-                any_jobs[pass] += any[pass][L] ? jobs[pass][L] : 0;
+                for (int j : jobs[pass][L]) {
+                    if (any[pass][L])
+                        any_jobs[pass] += j;
+                    else
+                        rest_launches[pass] +=
+                            (j + fft2d::kBatchTmaMaxJobs - 1) / fft2d::kBatchTmaMaxJobs;
+                }
             }
     }
     // every job of the pass's launch for any length, on stream s
@@ -636,34 +643,16 @@ fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in
         return any_jobs[pass] > fft2d::kBatchMaxJobs ? run_jobs(wide, pass, s)
                                                      : run_jobs(table, pass, s);
     };
-    fft2d_status result = FFT2D_OK;
-    if (!some_rest[0] && some_any[0])
-        result = run_any(FFT2D_PASS_ROWS, st);
-    if (result != FFT2D_OK)
-        return result;
-    if (!some_rest[0] && !some_rest[1])
-        return some_any[1] ? run_any(FFT2D_PASS_COLS, st) : FFT2D_OK;
-
-    BatchLanes *bl = batch_lanes(device, st);
-    if (!bl)
-        return FFT2D_ERR_OOM;
-    std::unique_lock<std::mutex> lanes_lock(bl->mu);
-    cudaError_t e = batch_lanes_prepare(*bl);
-    if (e == cudaSuccess)
-        e = lanes_wait_stream(*bl, st);
-    if (e != cudaSuccess)
-        return cuda_fail(e, "batch lanes");
-    int group = 0;
-    auto lane = [&] { return bl->s[group++ % kBatchLanes]; };
     // the groups of one length: a grouped launch, or (lines of 8192 and 16384
-    // points) each image's single-image pass, the same bits
-    auto run_rest = [&](int pass) {
+    // points) each image's single-image pass, the same bits; stream() gives
+    // each group its stream
+    auto run_rest = [&](int pass, auto stream) {
         const bool row = pass == FFT2D_PASS_ROWS;
         return batch_groups(
             n, plans, in, out, row,
             [&](int L) { return values[pass][L] > 0 && !any[pass][L]; },
             [&](fft2d::BatchTable &table, int L, int first) {
-                cudaStream_t ls = lane();
+                cudaStream_t ls = stream();
                 int *err = plans[first]->dev_err;
                 cudaError_t e = cudaSuccess;
                 if (L < 13) {
@@ -689,11 +678,36 @@ fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in
                 return e == cudaSuccess ? FFT2D_OK : cuda_fail(e, "batched pass");
             });
     };
+    fft2d_status result = FFT2D_OK;
+    if (!some_rest[0] && some_any[0])
+        result = run_any(FFT2D_PASS_ROWS, st);
+    if (result != FFT2D_OK)
+        return result;
+    if (!some_rest[0] && !some_rest[1])
+        return some_any[1] ? run_any(FFT2D_PASS_COLS, st) : FFT2D_OK;
+    // a column pass of one launch follows the rows on the caller's stream: with
+    // the rows there and the columns on a lane, the two changes of stream cost
+    // a batch of one 1024^2 image 17.5 us a call, and 21.3 once a larger batch
+    // had put work on the other lanes; this way 12.8
+    if (!some_rest[0] && !some_any[1] && rest_launches[1] == 1)
+        return run_rest(FFT2D_PASS_COLS, [st] { return st; });
+
+    BatchLanes *bl = batch_lanes(device, st);
+    if (!bl)
+        return FFT2D_ERR_OOM;
+    std::unique_lock<std::mutex> lanes_lock(bl->mu);
+    cudaError_t e = batch_lanes_prepare(*bl);
+    if (e == cudaSuccess)
+        e = lanes_wait_stream(*bl, st);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "batch lanes");
+    int group = 0;
+    auto lane = [&] { return bl->s[group++ % kBatchLanes]; };
     if (some_rest[0]) {
         if (some_any[0])
             result = run_any(FFT2D_PASS_ROWS, lane());
         if (result == FFT2D_OK)
-            result = run_rest(FFT2D_PASS_ROWS);
+            result = run_rest(FFT2D_PASS_ROWS, lane);
         if (result == FFT2D_OK && some_rest[1]) {
             // the column pass starts once every row group has finished
             e = stream_wait_lanes(*bl, bl->s[0]);
@@ -707,7 +721,7 @@ fft2d_status batched_run(int n, const fft2d_plan_t *plans, const void *const *in
         if (some_any[1])
             result = run_any(FFT2D_PASS_COLS, lane());
         if (result == FFT2D_OK)
-            result = run_rest(FFT2D_PASS_COLS);
+            result = run_rest(FFT2D_PASS_COLS, lane);
     }
     // the caller's stream waits for the lanes, after an error too
     e = stream_wait_lanes(*bl, st);

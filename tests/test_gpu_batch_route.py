@@ -57,3 +57,28 @@ def test_a_batch_of_many_images_shares_its_launches(n, want):
     for x, o in zip(xs, outs):
         s = tuple(x.shape)
         assert torch.equal(plans[s](x, one[s]), o)
+
+
+@pytest.mark.parametrize("shapes", [[(1024, 1024)], [(2048, 256)] * 4, [(1024, 512)] * 3 + [(1024, 1024)],
+                                    [(8192, 64)] * 2, [(1024, 512), (2048, 512)]])
+def test_columns_in_launches_of_their_own(shapes):
+    """Rows in the launch for any length and columns in one launch of their
+    own (which follows on the caller's stream) or in two (which do not): the
+    bits of each image's own transform, call after call on the same buffers."""
+    import paper_1505_08019_gb300 as fft
+    plans, handles, xs, outs = batch(shapes)
+    want = [plans[tuple(x.shape)](x) for x in xs]
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for _ in range(20):
+            for o in outs:
+                o.zero_()
+            fft.fft2d_exec_batched(handles, xs, outs)
+            fft.fft2d_exec_batched(handles, xs, outs)
+            got = [o.clone() for o in outs]
+    torch.cuda.synchronize()
+    assert all(torch.equal(g, w) for g, w in zip(got, want))
+    if shapes[0][0] < 8192:
+        assert len(launches(lambda s: fft.fft2d_exec_batched(handles, xs, outs, s))) \
+            == len({s[0] for s in shapes}) + 1
