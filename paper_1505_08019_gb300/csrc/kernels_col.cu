@@ -503,8 +503,9 @@ struct ColVariants {
     // as they fit the 152 SMs about once: the pass is then one CTA's latency.
     // 128 and 256 rows: "narrow" (4096 values) at every width, 2.6 / 3.2 us
     // and 3.0 / 4.2 for "plain" up to 2048 columns.  512 rows: "fine32g5"
-    // at every width, 2.9 / 3.5 us for "narrow" up to 1024 columns, 13.6 / 15.7
-    // at 8192: one exchange instead of two.  1024
+    // from a whole tile of 8 columns up, 2.9 / 3.5 us for "narrow" up to 1024
+    // columns, 13.6 / 15.7 at 8192: one exchange instead of two; in a tile that
+    // is partly empty its few threads take longer, 4.0 / 3.6 for 1 to 4.  1024
     // rows: "tma32g5", 3.3 against 4.9 us for "narrow" up to 512 columns, 8.9 /
     // 9.3 at 2048, 14.8 / 18.2 at 4096, 26.9 / 32.1 at 8192 (four CTAs per SM,
     // each with the next tile's first half on its way, against two that load,
@@ -527,7 +528,7 @@ struct ColVariants {
         if constexpr (L == 7 || L == 8)
             return index_of("narrow");
         else if constexpr (L == 9)
-            return index_of("fine32g5");
+            return index_of(cols < Fine5::W ? "narrow" : "fine32g5");
         else if constexpr (L == 10)
             return index_of(cols <= 8192 ? "tma32g5" : "tma64w8");
         else if constexpr (L == 11)

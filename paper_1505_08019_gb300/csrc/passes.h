@@ -304,8 +304,7 @@ cudaError_t launch_batch_any_h16(bool row, BatchTableH16 &t, int in_axis, cudaSt
 // Batches of equal images, this launch against a launch per length, at 2^21,
 // 2^22 and 2^23 values: 128^2 16 / 23, 26 / 48, 49 / 90 us; 256^2 14 / 22, 21 /
 // 32, 45 / 58; 512^2 16 / 27, 26 / 41, 52 / 67; 64x512 14 / 21, 22 / 28, 45 / 47;
-// 1024^2, where only the rows join, 23 / 25, 34 / 37, 61 / 60: even at the
-// limit.
+// 1024^2, where only the rows join, 17 / 23, 29 / 34, 56 / 59.
 // Rows run the CTAs of their own kernels.  Columns of up to 512 rows join, and
 // longer ones as long as the group fits 128 CTAs of 2^12 values
 // (col_small_tile): beyond that their 32-byte row segments lose to the wider

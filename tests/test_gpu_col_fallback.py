@@ -1,6 +1,6 @@
 """Column passes that TMA cannot feed (buffers of less than 16-byte alignment,
-fewer columns than a tile) run the kernel that serves their length best
-without it, with the plain kernel's bits."""
+fewer columns than a tile), or that fill no tile, run the kernel that serves
+their length best then, with the plain kernel's bits."""
 import pytest
 
 from _graph import launches
@@ -9,19 +9,23 @@ torch = pytest.importorskip("torch")
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="no CUDA GPU")]
 
 
-@pytest.mark.parametrize("cols,odd", [(1, 0), (2, 0), (4, 1), (8, 1), (64, 1), (1024, 1), (16384, 1)])
-def test_1024_rows_run_narrow_tiles(cols, odd):
+@pytest.mark.parametrize("rows,cols,odd", [(512, 1, 0), (512, 2, 0), (512, 4, 1), (1024, 1, 0), (1024, 2, 0),
+                                           (1024, 4, 1), (1024, 8, 1), (1024, 64, 1), (1024, 1024, 1),
+                                           (1024, 16384, 1)])
+def test_narrow_tiles(rows, cols, odd):
+    """512 rows: fewer columns than a tile of the default kernel; 1024 rows:
+    images that TMA cannot feed."""
     import paper_1505_08019_gb300 as fft
-    P = fft.FFT2D_PASS_COLS
-    names = [fft.fft2d_variant_name(P, 10, v) for v in range(fft.fft2d_variant_count(P, 10))]
-    buf = torch.view_as_complex(torch.randn(1024 * cols + 1, 2, device="cuda"))
-    x = buf[odd:odd + 1024 * cols].view(1024, cols)
+    P, L = fft.FFT2D_PASS_COLS, rows.bit_length() - 1
+    names = [fft.fft2d_variant_name(P, L, v) for v in range(fft.fft2d_variant_count(P, L))]
+    buf = torch.view_as_complex(torch.randn(rows * cols + 1, 2, device="cuda"))
+    x = buf[odd:odd + rows * cols].view(rows, cols)
 
     def geometry(p, out):
         fft.fft2d_exec_pass(p.handle, P, x, out)
         return launches(lambda s: fft.fft2d_exec_pass(p.handle, P, x, out, s))
 
-    with fft.Plan(1024, cols) as p:
+    with fft.Plan(rows, cols) as p:
         got, narrow, plain = (torch.empty_like(x) for _ in range(3))
         default = geometry(p, got)
         fft.fft2d_plan_set_variant(p.handle, P, names.index("narrow"))
